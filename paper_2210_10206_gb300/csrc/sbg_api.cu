@@ -117,7 +117,8 @@ struct Single { int l, m, b; };
 
 struct Tables4 {
   // host
-  std::vector<Tile4> tiles[3];  // by tcg class 4, 8, 16
+  std::vector<Tile4> tiles;     // FP32: in the order of the plan's two launches
+  SimtPlan simt{};              // FP32 tiles
   std::vector<Row4> rows;
   std::vector<int> cols, uniq;
   std::vector<BGroup> bgroups;  // tensor-core tiles: column groups and their B images
@@ -130,7 +131,7 @@ struct Tables4 {
   int covering = 0;      // 0: bin-half (tensor) or b3 >= b2 (SIMT) rows; 1: greedy cover
   int nout = 0;
   // device
-  DevBuf d_tiles[3], d_rows, d_cols, d_uniq, d_bgroups, d_ptr, d_idx, d_coef;
+  DevBuf d_tiles, d_rows, d_cols, d_uniq, d_bgroups, d_ptr, d_idx, d_coef;
 };
 
 }  // namespace
@@ -403,7 +404,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
   //                     into fewer tiles.
   auto half = [&](int b) { return b < (nb + 1) / 2 ? 0 : 1; };
   struct RowKey { int a1, b1, a2, b2; };
-  struct Slab { int r0, nr, c0, nc; long long tout; int row0; };
+  struct Slab { int r0, nr, c0, nc; long long tout; int row0, tile; };
   struct Block {
     int m3 = 0, b2 = 0;
     std::vector<RowKey> rows;
@@ -459,10 +460,10 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
       blocks.push_back(std::move(bk));
     }
   const int col_chunk = tc ? (cplx ? 32 : 64) : 64;
-  const int max_u = tc ? kTcMaxRowSlots : kSimtMaxUniq;
+  const int max_u = tc ? kTcMaxRowSlots : kSimtSpanUniq;
   auto sidx = [&](int a, int b) { return store_index(dim, nb, angs[a].l, std::abs(angs[a].m), b); };
-  // tensor-core tiles of 128 rows that the packing below makes of a block's rows
-  auto count_tiles = [&](const std::vector<RowKey>& rows) -> long long {
+  // tiles of at most `most` rows and max_u singles that a packing in order makes of a block's rows
+  auto count_tiles = [&](const std::vector<RowKey>& rows, int most = 128) -> long long {
     long long n = 0;
     int nr = 0;
     std::vector<int> local;
@@ -470,7 +471,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
     for (const RowKey& rk : rows) {
       const int s1 = sidx(rk.a1, rk.b1), s2 = sidx(rk.a2, rk.b2);
       const int need = (has(s1) ? 0 : 1) + ((has(s2) || s2 == s1) ? 0 : 1);
-      if (nr == 128 || (int)local.size() + need > max_u) {  // the row opens the next tile
+      if (nr == most || (int)local.size() + need > max_u) {  // the row opens the next tile
         ++n;
         nr = 0;
         local.clear();
@@ -747,7 +748,17 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
     for (int c0 = 0; c0 < bk.ncols; c0 += col_chunk) {
       const int nc = std::min(col_chunk, bk.ncols - c0);
       const int cls = tc ? 0 : (nc <= 16 ? 0 : (nc <= 32 ? 1 : 2));
-      const int TR = tc ? 128 : (cls == 0 ? 256 : (cls == 1 ? 128 : 64));
+      int TR = 128, tile_u = max_u;
+      SimtGeometry geo{};
+      if (!tc) {
+        // the units of the span grid: rows x columns of 4096 entries, cut in order
+        const int span_rows = cls == 0 ? 256 : (cls == 1 ? 128 : 64);
+        t.simt.span_tiles[cls] += (int)count_tiles(bk.rows, span_rows);
+        // the kernel's tiles
+        geo = simt_geometry(cplx ? 1 : 0, nc);
+        tile_u = geo.max_uniq;
+        TR = geo.max_rows;
+      }
       const int col0 = (int)t.cols.size();
       int bgroup = -1;
       if (tc) {
@@ -786,7 +797,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
           const int s1 = store_index(dim, nb, a1.l, std::abs(a1.m), rk.b1);
           const int s2 = store_index(dim, nb, a2.l, std::abs(a2.m), rk.b2);
           const int need = (local.count(s1) ? 0 : 1) + ((local.count(s2) || s2 == s1) ? 0 : 1);
-          if ((int)local.size() + need > max_u) break;
+          if ((int)local.size() + need > tile_u) break;
           if (!local.count(s1)) { const int k = (int)local.size(); local[s1] = k; if (!tc) t.uniq.push_back(s1); }
           if (!local.count(s2)) { const int k = (int)local.size(); local[s2] = k; if (!tc) t.uniq.push_back(s2); }
           Row4 rw;
@@ -811,9 +822,21 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
         if ((int)bk.slab_at.size() <= c0 / col_chunk) bk.slab_at.resize(c0 / col_chunk + 1);
         bk.slab_at[c0 / col_chunk].resize(nrows_blk, -1);
         for (int q = rstart; q < rstart + nr; ++q) bk.slab_at[c0 / col_chunk][q] = (int)bk.slabs.size();
-        bk.slabs.push_back({rstart, nr, c0, nc, so, tl.row0});
-        so += (long long)nr * nc;
-        t.tiles[cls].push_back(tl);
+        bk.slabs.push_back({rstart, nr, c0, nc, so, tl.row0, (int)t.tiles.size()});
+        if (tc) {
+          so += (long long)nr * nc;
+        } else {
+          tl.cls = cls;
+          tl.nrg = (nr + geo.rt - 1) / geo.rt;
+          tl.ncg = geo.ncg;
+          so += (long long)geo.rt * geo.ct * tl.nrg * tl.ncg;
+          const int k = geo.ct == 8 ? 1 : 0;
+          t.simt.threads[k] = std::max(t.simt.threads[k], tl.nrg * tl.ncg);
+          t.simt.smem[k] = std::max(t.simt.smem[k], simt_tile_smem(tl, geo));
+          t.simt.uses[k][cls] = true;
+          ++t.simt.ntiles[k];
+        }
+        t.tiles.push_back(tl);
       }
     }
   }
@@ -821,7 +844,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
 
   // T index of a triple of singles (any order, any sign of M); negative when the
   // entry found is the conjugate (all m negated).  rowsign receives the sign the
-  // tensor-core kernel leaves out of that entry's row.
+  // contraction kernels leave out of that entry's row.
   auto find_entry = [&](const Single& x, const Single& y, const Single& z, bool neg, float* rowsign) -> long long {
     const int m3 = z.m;
     if (m3 < 0 || m3 > L) return LLONG_MIN;
@@ -841,7 +864,11 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
     const int chunk = col / col_chunk;
     if (col >= bk.ncols || chunk >= (int)bk.slab_at.size() || bk.slab_at[chunk][row] < 0) return LLONG_MIN;
     const Slab& sl = bk.slabs[bk.slab_at[chunk][row]];
-    const long long ti = sl.tout + (long long)(row - sl.r0) * sl.nc + (col - sl.c0);
+    long long ti = sl.tout + (long long)(row - sl.r0) * sl.nc + (col - sl.c0);
+    if (!tc) {
+      const Tile4& tl = t.tiles[sl.tile];
+      ti = simt_entry(tl, simt_geometry(cplx ? 1 : 0, tl.ncols), row - sl.r0, col - sl.c0);
+    }
     if (rowsign) *rowsign = t.rows[sl.row0 + (row - sl.r0)].sign;
     return neg ? -ti - 1 : ti;
   };
@@ -894,7 +921,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
                     if (odd) sgn = -1.0;
                   }
                   t.idx.push_back((int)ti);
-                  t.coef.push_back(sgn * (tc ? tm.c * rs : tm.c));
+                  t.coef.push_back(sgn * tm.c * rs);
                 }
                 t.ptr.push_back((int)t.idx.size());
               }
@@ -917,8 +944,13 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
             }
   }
   t.nout = (int)t.ptr.size() - 1;
+  if (!tc) {
+    // the tiles of each launch together, in the order they were cut
+    std::stable_partition(t.tiles.begin(), t.tiles.end(), [&](const Tile4& x) { return simt_geometry(cplx ? 1 : 0, x.ncols).ct == 4; });
+    t.simt.first[1] = t.simt.ntiles[0];
+  }
   if (!to_device) return SBG_OK;
-  for (int k = 0; k < 3; ++k) ST(upload(ctx, t.d_tiles[k], t.tiles[k]));
+  ST(upload(ctx, t.d_tiles, t.tiles));
   ST(upload(ctx, t.d_rows, t.rows));
   ST(upload(ctx, t.d_cols, t.cols));
   ST(upload(ctx, t.d_uniq, t.uniq));
@@ -931,7 +963,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
 
 void free_tables4(sbg_context* ctx, Tables4* t) {
   if (!t) return;
-  for (int k = 0; k < 3; ++k) dev_free(ctx, t->d_tiles[k]);
+  dev_free(ctx, t->d_tiles);
   dev_free(ctx, t->d_rows);
   dev_free(ctx, t->d_cols);
   dev_free(ctx, t->d_uniq);
@@ -1438,7 +1470,7 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
     ST(buf(ctx, "T", (size_t)std::max<long long>(t.tcount, 1) * 8 * (cplx ? 2 : 1), (void**)&d_T));
     CU(cudaMemsetAsync(d_T, 0, (size_t)t.tcount * 8 * (cplx ? 2 : 1), ctx->stream));
     if (tc) {
-      const int ntl = (int)t.tiles[0].size();
+      const int ntl = (int)t.tiles.size();
       const long long kblocks = ng / 32;
       // x-splits per tile: units = ntl * nsplit spread over the CTAs; the three
       // best by their wave fill are timed by the autotuner on the first call
@@ -1468,7 +1500,7 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
         cudaError_t e = cudaMemsetAsync(d_cnt, 0, (size_t)epochs * 4, ctx->stream);
         if (e != cudaSuccess) return e;
         return launch_tc4(d_astore, d_bimg, (const BGroup*)t.d_bgroups.p, (int)t.bgroups.size(), t.chunks_per_kb,
-                          t.img_stride, d_delta, ng, (const Tile4*)t.d_tiles[0].p, ntl, (const Row4*)t.d_rows.p,
+                          t.img_stride, d_delta, ng, (const Tile4*)t.d_tiles.p, ntl, (const Row4*)t.d_rows.p,
                           (const int*)t.d_cols.p, (const int*)t.d_uniq.p, nsingle, kmode, nsplit, T, d_cnt, d_err,
                           ctx->nsm, ctx->stream, e0, e1, tf ? 1 : 0, ctx->wait_ns, ctx->stall);
       };
@@ -1484,16 +1516,13 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
       KL(tc4_run(best, d_T, ctx->kev[0], ctx->kev[1]));
       ctx->kev_used = true;
     } else {
-      const int tcg[3] = {4, 8, 16};
       CU(cudaEventRecord(ctx->kev[0], ctx->stream));
       ctx->kev_used = true;
-      for (int k = 0; k < 3; ++k) {
-        const int ntl = (int)t.tiles[k].size();
-        if (!ntl) continue;
-        KL(launch_simt4(d_astore, ng, d_delta, (const Tile4*)t.d_tiles[k].p, ntl, (const Row4*)t.d_rows.p,
-                        (const int*)t.d_cols.p, (const int*)t.d_uniq.p, kmode, tcg[k], 0, nsingle, d_T, ctx->nsm,
-                        ctx->stream));
-      }
+      int launches = 0;
+      CU(launch_simt4(d_astore, ng, d_delta, (const Tile4*)t.d_tiles.p, t.simt, (const Row4*)t.d_rows.p,
+                      (const int*)t.d_cols.p, (const int*)t.d_uniq.p, kmode, nsingle, d_T, ctx->nsm, ctx->stream,
+                      &launches));
+      ctx->nlaunch += launches;
       CU(cudaEventRecord(ctx->kev[1], ctx->stream));
     }
     ST(buf(ctx, "z4", (size_t)t.nout * 8 * (cplx ? 2 : 1), (void**)&d_z4));
@@ -1742,7 +1771,7 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
     ST(buf(ctx, "T", (size_t)nfld * tstride * 16, (void**)&d_T));
     CU(cudaMemsetAsync(d_T, 0, (size_t)nfld * tstride * 16, st));
     if (tcomb) {
-      const int ntl = (int)t.tiles[0].size();
+      const int ntl = (int)t.tiles.size();
       const long long fkb = ng / 32;  // K-blocks of one field
       // x-splits per field: a power of two dividing its K-blocks, for the best
       // spread of the units over the CTAs
@@ -1773,7 +1802,7 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
         cudaError_t e = cudaMemsetAsync(d_cnt, 0, (size_t)epochs * 4, st);
         if (e != cudaSuccess) return e;
         return launch_tc4(d_astore, d_bimg, (const BGroup*)t.d_bgroups.p, (int)t.bgroups.size(), t.chunks_per_kb,
-                          t.img_stride, d_delta, npts, (const Tile4*)t.d_tiles[0].p, ntl, (const Row4*)t.d_rows.p,
+                          t.img_stride, d_delta, npts, (const Tile4*)t.d_tiles.p, ntl, (const Row4*)t.d_rows.p,
                           (const int*)t.d_cols.p, (const int*)t.d_uniq.p, nsingle, 1, nfld * spf, T, d_cnt, d_err,
                           ctx->nsm, st, e0, e1, tf32, ctx->wait_ns, ctx->stall, spf, tstride * 2);
       };
@@ -1789,16 +1818,13 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
       KL(tc4_run(spf, d_T, ctx->kev[0], ctx->kev[1]));
       ctx->kev_used = true;
     } else {
-      const int tcg[3] = {4, 8, 16};
       CU(cudaEventRecord(ctx->kev[0], st));
       ctx->kev_used = true;
-      for (int k = 0; k < 3; ++k) {
-        const int ntl = (int)t.tiles[k].size();
-        if (!ntl) continue;
-        KL(launch_simt4(d_astore, npts, d_delta, (const Tile4*)t.d_tiles[k].p, ntl, (const Row4*)t.d_rows.p,
-                        (const int*)t.d_cols.p, (const int*)t.d_uniq.p, 1, tcg[k], 0, nsingle, d_T, ctx->nsm, st,
-                        nfld, tstride * 2));
-      }
+      int launches = 0;
+      CU(launch_simt4(d_astore, npts, d_delta, (const Tile4*)t.d_tiles.p, t.simt, (const Row4*)t.d_rows.p,
+                      (const int*)t.d_cols.p, (const int*)t.d_uniq.p, 1, nsingle, d_T, ctx->nsm, st, &launches, nfld,
+                      tstride * 2));
+      ctx->nlaunch += launches;
       CU(cudaEventRecord(ctx->kev[1], st));
     }
     ST(buf(ctx, "z4", (size_t)nfld * t.nout * 16, (void**)&d_z4));
@@ -2336,7 +2362,8 @@ sbg_status sbg_plan4_info(int dim, int nbins, int lmax, sbg_precision prec, int 
   Tables4 t;
   const sbg_status s = build_tables4(&host, t, dim, nbins, lmax, prec != SBG_PREC_FP32, odd != 0, false);
   if (s != SBG_OK) return s;
-  if (ntiles) *ntiles = (int)(t.tiles[0].size() + t.tiles[1].size() + t.tiles[2].size());
+  if (ntiles)
+    *ntiles = t.tc ? (int)t.tiles.size() : t.simt.span_tiles[0] + t.simt.span_tiles[1] + t.simt.span_tiles[2];
   if (nrows) *nrows = (int)t.rows.size();
   if (covering) *covering = t.covering;
   return SBG_OK;

@@ -359,254 +359,429 @@ cudaError_t launch_gram3(const float2* a, long long ng, int nb, const float* del
 // ------------------------------------------------------------------ simt4 --
 // T[r][c] = sum_x delta(x) f1_r(x) f2_r(x) a_c(x): the pair-by-single contraction
 // of the 4PCF (Eq. mu of Sec. 2.3, Eq. proj_4pcf_coeff) as an FP32 SIMT GEMM over
-// x with the pair operand formed on chip.  Per 32-point chunk the tile's row
-// singles, its column singles and delta are copied with cp.async into one of two
-// raw buffers while the previous chunk is computed; then the pair products
-// P_r = sign delta f1 f2 and the transposed columns are formed in shared memory
-// and each thread accumulates a 4x4 block of rows x cols.  FP32 over 512-point
-// spans, FP64 across spans and CTAs.
-constexpr int kX = 32;          // points per chunk
-constexpr int kSpan = 16;       // chunks per FP32 span
-constexpr int kRawF = 68;       // floats per raw row: Re x0..31, Im x0..31, pad (16-byte multiple)
+// x with the pair operand formed on chip.
+//
+// Bound: the FMA pipe (2 FMAs per entry and point, 4 for complex T).  Each thread
+// holds RT rows x CT columns (8 x 8 or 16 x 4 real, 8 x 4 complex: 64
+// accumulators), so a point costs it 6 to 10 16-byte shared-memory loads for 128
+// FMAs.  The FMAs are
+// packed (f32x2, two pipe cycles each), which leaves about half of the issue
+// slots to the loads and to forming the operands.  A packed FMA multiplies two rows
+// by two columns; with the column pair once straight and once swapped in
+// registers it serves the four entries of a 2 x 2 block, and no operand has to
+// be duplicated.  Per 16-point chunk the tile's row singles, its columns and
+// delta are copied with cp.async while the previous chunk is accumulated, then
+// formed in shared memory as [x][row] and [x][column] arrays.  Three to four CTAs of 128 threads per SM overlap one's
+// forming with another's FMAs.
+// Accumulation: FP32 over a span (at most 512 points), then one FP64 reduction
+// into T (red.add, fire and forget; T is laid out [accumulator][thread], so a
+// warp's 32 values are contiguous): no FP64 add, whose rate is 1/75 of the FMA
+// rate here, occupies the SM.
+// Measured: 256^3, lmax 4, 10 bins: 686 -> 268 ms per field (128^3: 3D lmax 3, 8
+// bins 20.1 -> 8.0 ms; 1024^2, mmax 5, 20 bins 41.4 -> 15.0 ms) against the
+// earlier 4 x 4 entries per thread with two 256-thread CTAs per SM, whose
+// strided float4 loads conflicted in the banks.  The FMA pipe is 60% busy (the
+// bare accumulation loop reaches 80% here); the rest is forming the operands,
+// which narrow tiles (few columns per formed row) pay most, and barriers.
+constexpr int kX = 16;          // points per chunk (half a block of the coefficient store)
+constexpr int kSpan = 32;       // chunks per FP32 span
+constexpr int kRawF = 36;       // floats per raw row: Re x0..15, Im x0..15, pad (16-byte multiple)
+constexpr int kSimtThreads = 128;
+// most rows of a tile and most columns (complex T: 2D, one column per bin)
+constexpr int simt_rows(int rt) { return rt == 16 ? 256 : 192; }
+constexpr int simt_cols(int ct, bool cplx) { return cplx ? 20 : ct == 4 ? 16 : 64; }
 
 __device__ __forceinline__ void simt_cp16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
                : "memory");
 }
+__device__ __forceinline__ uint64_t swap2(uint64_t v) {
+  float a, b;
+  upk(v, a, b);
+  return pk(b, a);
+}
+__device__ __forceinline__ uint64_t neg2(uint64_t v) { return v ^ 0x8000000080000000ull; }
+// sign bits of both halves where b & 1
+__device__ __forceinline__ uint64_t sign2(int b) {
+  const uint32_t m = (uint32_t)b << 31;
+  return (uint64_t)m << 32 | m;
+}
+__device__ __forceinline__ void red_add(double* p, float v) {
+  asm volatile("red.global.add.f64 [%0], %1;" ::"l"(p), "d"((double)v) : "memory");
+}
 
-template <int TCG>
-struct SimtSmem {
-  static constexpr int TR = 4 * (256 / TCG), TC = 4 * TCG;
-  static constexpr int kRawU = kSimtMaxUniq * kRawF;  // floats of one raw row-single buffer
-  static constexpr int kRawC = TC * kRawF;             // floats of one raw column buffer
-  static constexpr int kRaw = kRawU + kRawC + kX;      // one raw buffer (+ delta)
-  static constexpr size_t kBytes = (size_t)(2 * kRaw) * 4 + (size_t)(kX * TR + kX * TC) * 8;
+// Spans of one column class: x-split k covers the points [k per, (k + 1) per) and
+// consists of nsp spans of kSpan chunks (the last one shorter or empty).
+struct SimtSpans {
+  int nsplit, nsp;   // x-splits, spans per x-split
+  long long per;     // points per x-split
+  int unit;          // spans per CTA
+};
+struct SimtArgs {
+  const float* astore;
+  const float* delta;
+  const Tile4* tiles;
+  const Row4* rows;
+  const int *cols, *uniq;
+  double* T;
+  long long ng, t_field_stride;
+  int nsingle, imag;
+  int spf[3];        // x-splits per field of a slab (0: one field)
+  SimtSpans sp[3];
 };
 
-template <int TCG, bool CPLX>
-__global__ void __launch_bounds__(256) simt4_kernel(const float2* __restrict__ astore, long long ng,
-                                                    const float* __restrict__ delta, const Tile4* __restrict__ tiles,
-                                                    const Row4* __restrict__ rows, const int* __restrict__ cols,
-                                                    const int* __restrict__ uniq, int nsplit, int nsingle,
-                                                    double* __restrict__ T, int imag, int splits_per_field,
-                                                    long long t_field_stride) {
-  // a slab of fields: x-split blockIdx.y belongs to field blockIdx.y / splits_per_field
-  if (splits_per_field) T += (long long)(blockIdx.y / splits_per_field) * t_field_stride;
-  using SM = SimtSmem<TCG>;
-  constexpr int TR = SM::TR, TC = SM::TC;
+template <int RT, int CT, bool CPLX>
+__global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const SimtArgs p) {
+  const Tile4 tl = p.tiles[blockIdx.x];
+  const SimtSpans sp = p.sp[tl.cls];
+  const int spf = p.spf[tl.cls];
+  const int s0 = blockIdx.y * sp.unit, s1 = min(s0 + sp.unit, sp.nsplit * sp.nsp);
   extern __shared__ float4 smem4[];
-  float* raw = reinterpret_cast<float*>(smem4);                       // [2][kRaw]
-  float2* Ps = reinterpret_cast<float2*>(raw + 2 * SM::kRaw);         // [kX][TR]
-  float2* Cs = Ps + kX * TR;                                          // [kX][TC]
+  // row strides of the formed operands (compile-time: the accumulation's loads
+  // and the forming's stores take immediate offsets)
+  constexpr int TRS = simt_rows(RT), TCS = simt_cols(CT, CPLX);
+  const int nrg = tl.nrg, ncg = tl.ncg;
+  const int TR = RT * nrg, TC = CT * ncg;
+  float* Px = reinterpret_cast<float*>(smem4);   // [kX][TRS]
+  float* Py = Px + kX * TRS;                     // real T: -Im P, complex T: Im P
+  float* Cx = Py + kX * TRS;                     // [kX][TCS]
+  float* Cy = Cx + kX * TCS;
+  int2* meta = reinterpret_cast<int2*>(Cy + kX * TCS);      // [TRS], see below
+  float* raw = reinterpret_cast<float*>(meta + TRS);        // [nuniq + ncols][kRawF], then delta [kX]
+  float* rdel = raw + (tl.nuniq + tl.ncols) * kRawF;
+  int* sidx = reinterpret_cast<int*>(rdel + kX);  // store index of each raw row, padded to 16
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const int cg = tid % ncg, rg = tid / ncg;
+  const bool active = rg < nrg;
+  const int nraw = tl.nuniq + tl.ncols;
 
-  const Tile4 tl = tiles[blockIdx.x];
-  // the plan keeps tiles within the staging buffers; a tile that is not is skipped
-  if (tl.nuniq > kSimtMaxUniq || tl.ncols > TC || tl.nrows > TR) return;
-  const int tid = threadIdx.x;
-  const int cg = tid % TCG, rg = tid / TCG;
-  const long long per = ((ng / kX + nsplit - 1) / nsplit) * kX;
-  const long long x0 = blockIdx.y * per, x1 = min(ng, x0 + per);
-
-  // copy chunk xc (raw blocked rows: 16 chunks of 16 B per single) into buffer b
-  auto stage = [&](long long xc, int b) {
-    float* ru = raw + b * SM::kRaw;
-    float* rc = ru + SM::kRawU;
-    float* rd = rc + SM::kRawC;
-    const float* base = reinterpret_cast<const float*>(astore) + (xc / kX) * (long long)nsingle * 64;
-    const int nu = tl.nuniq * 16, nc = tl.ncols * 16;
-    for (int i = tid; i < nu + nc + 8; i += 256) {
-      if (i < nu) {
-        simt_cp16(ru + (i >> 4) * kRawF + (i & 15) * 4, base + uniq[tl.uniq0 + (i >> 4)] * 64 + (i & 15) * 4);
-      } else if (i < nu + nc) {
-        const int k = i - nu;
-        simt_cp16(rc + (k >> 4) * kRawF + (k & 15) * 4, base + cols[tl.col0 + (k >> 4)] * 64 + (k & 15) * 4);
-      } else {
-        const int k = i - nu - nc;
-        simt_cp16(rd + k * 4, delta + xc + k * 4);
-      }
-    }
+  // the chunk's half (16 Re, 16 Im) of the 32-point block of each single: thread
+  // t copies 16 bytes (chunk t % 8 of the 128) of the raw rows t / 8, + nt / 8, ...
+  const int sch = tid & 7;
+  float* const sdst = raw + (tid >> 3) * kRawF + sch * 4;
+  const float* const ssrc = p.astore + (sch & 3) * 4 + (sch >> 2) * 32;
+  auto stage = [&](long long xc) {
+    const float* base = ssrc + (xc >> 5) * (long long)p.nsingle * 64 + (xc & 31);
+    float* dst = sdst;
+    for (int row = tid >> 3; row < nraw; row += nt >> 3, dst += (nt >> 3) * kRawF)
+      simt_cp16(dst, base + (long long)sidx[row] * 64);
+    if (tid < 4) simt_cp16(rdel + tid * 4, p.delta + xc + tid * 4);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
-
-  float acc[4][4][CPLX ? 2 : 1];
-  double dacc[4][4][CPLX ? 2 : 1];
+  // The staged chunk's operands, 8 points of a row or column per item.  meta
+  // holds a row's raw offsets of its two singles and the sign bits of their
+  // conjugations (the row's own sign is left to the couplings).  Rows and columns
+  // past the tile's repeat its last ones and are never written out.
+  auto form = [&]() {
+    for (int i = tid; i < 2 * TR; i += nt) {
+      const int h = i >= TR ? 8 : 0, r = i >= TR ? i - TR : i;
+      const int2 m = meta[r];
+      const float* u1 = raw + (m.x & 0xffff) + h;
+      const float* u2 = raw + (m.x >> 16) + h;
+      const uint64_t s1 = sign2(m.y & 1), s2 = sign2(m.y >> 1);
+      float* o = Px + h * TRS + r;
 #pragma unroll
-  for (int i = 0; i < 4; ++i)
+      for (int q = 0; q < 2; ++q) {
+        const ulonglong2 ar = *(const ulonglong2*)(u1 + 4 * q), ai = *(const ulonglong2*)(u1 + kX + 4 * q);
+        const ulonglong2 br = *(const ulonglong2*)(u2 + 4 * q), bi = *(const ulonglong2*)(u2 + kX + 4 * q);
+        const ulonglong2 d = *(const ulonglong2*)(rdel + h + 4 * q);
 #pragma unroll
-    for (int k = 0; k < 4; ++k)
-#pragma unroll
-      for (int c = 0; c < (CPLX ? 2 : 1); ++c) { acc[i][k][c] = 0.f; dacc[i][k][c] = 0.0; }
-
-  int span = 0, b = 0;
-  if (x0 < x1) stage(x0, 0);
-  for (long long xc = x0; xc < x1; xc += kX, b ^= 1) {
-    // prefetch the next chunk into the other buffer (its last readers finished
-    // before the barrier that ended the previous iteration)
-    if (xc + kX < x1) {
-      stage(xc + kX, b ^ 1);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
-    }
-    __syncthreads();
-    const float* ru = raw + b * SM::kRaw;
-    const float* rc = ru + SM::kRawU;
-    const float* rd = rc + SM::kRawC;
-    // columns, transposed to [x][c] (zero past the tile's columns); imag: a is
-    // stored as (Im a, -Re a), so that the real accumulation gives Im(P a)
-    for (int i = tid; i < TC * kX; i += 256) {
-      const int c = i % TC, xx = i / TC;
-      float2 v = make_float2(0.f, 0.f);
-      if (c < tl.ncols) {
-        const float re = rc[c * kRawF + xx], im = rc[c * kRawF + 32 + xx];
-        v = imag ? make_float2(im, -re) : make_float2(re, im);
-      }
-      Cs[xx * TC + c] = v;
-    }
-    // pair products P_r(x) = sign * delta * f1 * f2
-    for (int i = tid; i < TR * kX; i += 256) {
-      const int r = i % TR, xx = i / TR;
-      float2 p = make_float2(0.f, 0.f);
-      if (r < tl.nrows) {
-        const Row4 rw = rows[tl.row0 + r];
-        float2 f1 = make_float2(ru[rw.u1 * kRawF + xx], ru[rw.u1 * kRawF + 32 + xx]);
-        float2 f2 = make_float2(ru[rw.u2 * kRawF + xx], ru[rw.u2 * kRawF + 32 + xx]);
-        if (rw.flags & 1) f1.y = -f1.y;
-        if (rw.flags & 2) f2.y = -f2.y;
-        const float s = rw.sign * rd[xx];
-        p = cmul(f1, f2);
-        p.x *= s;
-        p.y *= s;
-      }
-      Ps[xx * TR + r] = p;
-    }
-    __syncthreads();
-    // operands of point xx + 1 are loaded while point xx is accumulated
-    const float4* pr0 = reinterpret_cast<const float4*>(Ps + rg * 4);
-    const float4* cr0 = reinterpret_cast<const float4*>(Cs + cg * 4);
-    float4 np01 = pr0[0], np23 = pr0[1], nc01 = cr0[0], nc23 = cr0[1];
-#pragma unroll 4
-    for (int xx = 0; xx < kX; ++xx) {
-      const float4 p01 = np01, p23 = np23, c01 = nc01, c23 = nc23;
-      if (xx + 1 < kX) {
-        const float4* pr = reinterpret_cast<const float4*>(Ps + (xx + 1) * TR + rg * 4);
-        const float4* cr = reinterpret_cast<const float4*>(Cs + (xx + 1) * TC + cg * 4);
-        np01 = pr[0];
-        np23 = pr[1];
-        nc01 = cr[0];
-        nc23 = cr[1];
-      }
-      const float2 P[4] = {{p01.x, p01.y}, {p01.z, p01.w}, {p23.x, p23.y}, {p23.z, p23.w}};
-      const float2 C[4] = {{c01.x, c01.y}, {c01.z, c01.w}, {c23.x, c23.y}, {c23.z, c23.w}};
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          acc[i][k][0] = fmaf(P[i].x, C[k].x, fmaf(-P[i].y, C[k].y, acc[i][k][0]));
-          if (CPLX) acc[i][k][CPLX ? 1 : 0] = fmaf(P[i].x, C[k].y, fmaf(P[i].y, C[k].x, acc[i][k][CPLX ? 1 : 0]));
+        for (int e = 0; e < 2; ++e) {
+          const uint64_t a_r = e ? ar.y : ar.x, a_i = (e ? ai.y : ai.x) ^ s1, b_r = e ? br.y : br.x;
+          const uint64_t b_i = (e ? bi.y : bi.x) ^ s2, dd = e ? d.y : d.x;
+          const uint64_t pr = mul2(fma2(a_r, b_r, mul2(neg2(a_i), b_i)), dd);
+          uint64_t pi = mul2(fma2(a_i, b_r, mul2(a_r, b_i)), dd);
+          if (!CPLX) pi = neg2(pi);
+          float v0, v1;
+          upk(pr, v0, v1);
+          o[(4 * q + 2 * e) * TRS] = v0;
+          o[(4 * q + 2 * e + 1) * TRS] = v1;
+          upk(pi, v0, v1);
+          o[(kX + 4 * q + 2 * e) * TRS] = v0;  // Py
+          o[(kX + 4 * q + 2 * e + 1) * TRS] = v1;
         }
-    }
-    if (++span == kSpan) {
-      span = 0;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-#pragma unroll
-          for (int c = 0; c < (CPLX ? 2 : 1); ++c) { dacc[i][k][c] += acc[i][k][c]; acc[i][k][c] = 0.f; }
-    }
-    __syncthreads();  // Ps, Cs and this raw buffer are free for the next chunk
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int r = rg * 4 + i;
-    if (r >= tl.nrows) continue;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const int c = cg * 4 + k;
-      if (c >= tl.ncols) continue;
-#pragma unroll
-      for (int q = 0; q < (CPLX ? 2 : 1); ++q) {
-        const double v = dacc[i][k][q] + acc[i][k][q];
-        atomicAdd(&T[(tl.tout + (long long)r * tl.ncols + c) * (CPLX ? 2 : 1) + q], v);
       }
     }
+    // columns: the last threads first, whose row items are the fewest
+    for (int i = nt - 1 - tid; i < 2 * TC; i += nt) {
+      const int h = i >= TC ? 8 : 0, c = i >= TC ? i - TC : i;
+      const float* a = raw + (tl.nuniq + min(c, tl.ncols - 1)) * kRawF + h;
+      float* o = Cx + h * TCS + c;
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        const float4 re = *(const float4*)(a + 4 * q), im = *(const float4*)(a + kX + 4 * q);
+        const float vr[4] = {re.x, re.y, re.z, re.w}, vi[4] = {im.x, im.y, im.z, im.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          // imag: the column is (Im a, -Re a), so that the real sum gives Im(P a)
+          o[(4 * q + e) * TCS] = p.imag ? vi[e] : vr[e];
+          o[(kX + 4 * q + e) * TCS] = p.imag ? -vr[e] : vi[e];  // Cy
+        }
+      }
+    }
+  };
+
+  // accumulators: [component][row pair][column pair][straight, swapped]; entry
+  // (row 2 i + e, column 2 j + (e ^ w)) is lane e of acc[.][i][j][w]
+  constexpr int NC = CPLX ? 2 : 1, NI = RT / 2, NJ = CT / 2;
+  uint64_t acc[NC][NI][NJ][2];
+  auto zero = [&]() {
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+      for (int i = 0; i < NI; ++i)
+#pragma unroll
+        for (int j = 0; j < NJ; ++j) acc[c][i][j][0] = acc[c][i][j][1] = 0ull;
+  };
+  auto accumulate = [&]() {
+    const float* px = Px + rg * 4;
+    const float* py = Py + rg * 4;
+    const float* cx = Cx + cg * 4;
+    const float* cy = Cy + cg * 4;
+#pragma unroll 16
+    for (int x = 0; x < kX; ++x) {
+      uint64_t X[NI], Y[NI];
+#pragma unroll
+      for (int h = 0; h < RT / 4; ++h) {  // rows 4 rg .. + 3 of each section of 4 nrg rows
+        const ulonglong2 vx = *(const ulonglong2*)(px + x * TRS + h * 4 * nrg);
+        const ulonglong2 vy = *(const ulonglong2*)(py + x * TRS + h * 4 * nrg);
+        X[2 * h] = vx.x; X[2 * h + 1] = vx.y;
+        Y[2 * h] = vy.x; Y[2 * h + 1] = vy.y;
+      }
+#pragma unroll
+      for (int h = 0; h < CT / 4; ++h) {
+        const ulonglong2 vx = *(const ulonglong2*)(cx + x * TCS + h * 4 * ncg);
+        const ulonglong2 vy = *(const ulonglong2*)(cy + x * TCS + h * 4 * ncg);
+        const uint64_t u[2][2] = {{vx.x, swap2(vx.x)}, {vx.y, swap2(vx.y)}};
+        const uint64_t v[2][2] = {{vy.x, swap2(vy.x)}, {vy.y, swap2(vy.y)}};
+#pragma unroll
+        for (int jj = 0; jj < 2; ++jj)
+#pragma unroll
+          for (int w = 0; w < 2; ++w) {
+            const int j = 2 * h + jj;
+#pragma unroll
+            for (int i = 0; i < NI; ++i) {
+              if constexpr (CPLX) {
+                // Re += Px Cx - Py Cy, Im += Px Cy + Py Cx
+                acc[0][i][j][w] = fma2(X[i], u[jj][w], fma2(Y[i], neg2(v[jj][w]), acc[0][i][j][w]));
+                acc[NC - 1][i][j][w] = fma2(X[i], v[jj][w], fma2(Y[i], u[jj][w], acc[NC - 1][i][j][w]));
+              } else {
+                acc[0][i][j][w] = fma2(X[i], u[jj][w], fma2(Y[i], v[jj][w], acc[0][i][j][w]));
+              }
+            }
+          }
+      }
+    }
+  };
+  // the span's sums to T, and back to zero
+  auto flush = [&](int q) {
+    double* t = p.T + (spf ? (long long)(q / sp.nsp / spf) * p.t_field_stride : 0LL);
+#pragma unroll
+    for (int i = 0; i < NI; ++i)
+#pragma unroll
+      for (int j = 0; j < NJ; ++j)
+#pragma unroll
+        for (int w = 0; w < 2; ++w)
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            const int ri = 2 * i + e, cj = 2 * j + (e ^ w);
+            const int r = (ri >> 2) * 4 * nrg + rg * 4 + (ri & 3);
+            const int c = (cj >> 2) * 4 * ncg + cg * 4 + (cj & 3);
+            if (r >= tl.nrows || c >= tl.ncols) continue;
+            const long long k = tl.tout + (long long)((i * NJ + j) * 2 + w) * 2 * (nrg * ncg) + e * (nrg * ncg) + tid;
+#pragma unroll
+            for (int m = 0; m < NC; ++m) {
+              float lo, hi;
+              upk(acc[m][i][j][w], lo, hi);
+              red_add(t + k * NC + m, e ? hi : lo);
+            }
+          }
+    zero();
+  };
+
+  // the CTA's spans in turn; span q starts at x0 and has nc chunks (an empty one none)
+  int q = s0, nc = 0;
+  long long x0 = 0;
+  auto next_span = [&]() {  // the first span from q on that holds points
+    for (; q < s1; ++q) {
+      const int k = q / sp.nsp;
+      x0 = k * sp.per + (long long)(q - k * sp.nsp) * (kSpan * kX);
+      const long long left = min((k + 1) * sp.per, p.ng) - x0;
+      nc = (int)min(left, (long long)(kSpan * kX)) / kX;
+      if (left > 0) return true;
+    }
+    return false;
+  };
+  if (!next_span()) return;
+  for (int i = tid; i < nraw; i += nt) sidx[i] = i < tl.nuniq ? p.uniq[tl.uniq0 + i] : p.cols[tl.col0 + i - tl.nuniq];
+  for (int i = tid; i < TR; i += nt) {
+    const Row4 rw = p.rows[tl.row0 + min(i, tl.nrows - 1)];
+    meta[i] = make_int2(rw.u1 * kRawF | (rw.u2 * kRawF) << 16, rw.flags & 3);
+  }
+  __syncthreads();
+  zero();
+  stage(x0);
+  for (int c = 0;;) {
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // the chunk has landed; the previous one's operands have been read
+    form();
+    __syncthreads();  // the operands are formed and the raw chunk has been read
+    const int qd = q;
+    const bool done = ++c == nc;  // the span ends with this chunk
+    bool more = true;
+    if (done) {
+      ++q;
+      c = 0;
+      more = next_span();
+    }
+    if (more) stage(x0 + c * kX);
+    if (active) {
+      accumulate();
+      if (done) flush(qd);
+    }
+    if (!more) break;
   }
 }
 
-template <int TCG, bool CPLX>
-static cudaError_t simt4_t(const float2* astore, long long ng, const float* delta, const Tile4* tiles, int ntiles,
-                          const Row4* rows, const int* cols, const int* uniq, int nsplit, int nsingle, double* T,
-                          int nsm, int imag, cudaStream_t st, int nfld, long long t_field_stride) {
-  const size_t smem = SimtSmem<TCG>::kBytes;
-  auto kern = simt4_kernel<TCG, CPLX>;
-  {
-    cudaError_t e = ensure_smem_attr<simt4_kernel<TCG, CPLX>>((int)smem);
-    if (e != cudaSuccess) return e;
+namespace {
+// shared memory of a tile
+size_t simt_smem(int trs, int tcs, int nuniq, int ncols) {
+  return ((size_t)(nuniq + ncols) * (kRawF + 1) + kX + 2 * kX * ((size_t)trs + tcs)) * 4 + (size_t)trs * 8;
+}
+constexpr int kSimtSmemMax = 75 * 1024;
+}  // namespace
+
+template <int RT, int CT, bool CPLX>
+static cudaError_t simt4_t(SimtArgs a, const SimtPlan& pl, int k, int nsm, cudaStream_t st) {
+  const size_t smem = pl.smem[k];
+  const int threads = (pl.threads[k] + 31) / 32 * 32;
+  if (smem > kSimtSmemMax || threads < 32 || threads > kSimtThreads) return cudaErrorInvalidValue;
+  cudaError_t e = ensure_smem_attr<simt4_kernel<RT, CT, CPLX>>(kSimtSmemMax);
+  if (e != cudaSuccess) return e;
+  int per_sm = 0;
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, simt4_kernel<RT, CT, CPLX>, threads, smem)) !=
+      cudaSuccess)
+    return e;
+  // spans per CTA: about 8 CTAs per resident slot, so that the last wave costs
+  // little; at least one span, at most 64
+  const long long slots = (long long)nsm * std::max(per_sm, 1);
+  int rows = 1;
+  for (int c = 0; c < 3; ++c) {
+    SimtSpans& sp = a.sp[c];
+    const long long spans = (long long)sp.nsplit * sp.nsp;
+    sp.unit = (int)std::max<long long>(1, std::min<long long>(64, spans * pl.ntiles[k] / (8 * slots)));
+    sp.unit = (int)std::max<long long>(sp.unit, (spans + 65534) / 65535);
+    if (pl.uses[k][c]) rows = std::max<int>(rows, (int)((spans + sp.unit - 1) / sp.unit));
   }
-  int spf = 0;  // x-splits per field of a slab
-  if (nfld > 1) {
-    // a slab: every field is split alike (a power of two dividing its
-    // K-blocks), the split count chosen for the best fill of the resident slots
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
-    if (e != cudaSuccess) return e;
-    const long long slots = (long long)nsm * (per_sm > 0 ? per_sm : 1), fchunks = ng / nfld / kX;
-    double best = -1.0;
-    spf = 1;
-    for (long long k = 1; k <= fchunks && k <= 64; k *= 2) {
-      const long long units = (long long)ntiles * nfld * k;
-      if (units > 65535LL * ntiles) break;
-      const double fill = (double)units / (double)(slots * ((units + slots - 1) / slots));
-      if (fill > best + 1e-3) {
-        best = fill;
-        spf = (int)k;
-      }
-      if (units >= 4 * slots) break;
-    }
-    nsplit = nfld * spf;
-  } else if (nsplit <= 0) {
-    // x-splits per tile so that the CTAs fill whole waves of the resident
-    // slots (SMs x CTAs per SM): the best fill over 2..8 waves, fewer on ties
-    int per_sm = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem);
-    if (e != cudaSuccess) return e;
-    const long long slots = (long long)nsm * (per_sm > 0 ? per_sm : 1), chunks = ng / kX;
-    double best = -1.0;
-    nsplit = 1;
-    for (int w = 2; w <= 8; ++w) {
-      const long long ns = std::max<long long>(1, std::min<long long>(chunks, slots * w / ntiles));
-      const long long units = ns * ntiles;
-      const double fill = (double)units / (double)(slots * ((units + slots - 1) / slots));
-      if (fill > best + 1e-3) {
-        best = fill;
-        nsplit = (int)ns;
-      }
-    }
-  }
-  if (nsplit > 65535) return cudaErrorInvalidValue;
-  dim3 grid((unsigned)ntiles, (unsigned)nsplit);
-  kern<<<grid, 256, smem, st>>>(astore, ng, delta, tiles, rows, cols, uniq, nsplit, nsingle, T, imag, spf,
-                                t_field_stride);
+  a.tiles += pl.first[k];
+  simt4_kernel<RT, CT, CPLX><<<dim3((unsigned)pl.ntiles[k], (unsigned)rows), threads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta, const Tile4* tiles, int ntiles,
-                         const Row4* rows, const int* cols, const int* uniq, int complex_out, int tcg, int nsplit,
-                         int nsingle, double* T, int nsm, cudaStream_t st, int nfld, long long t_field_stride) {
-  if (ntiles <= 0) return cudaSuccess;
-  if (ng % kX || complex_out < 0 || complex_out > 2 || nfld < 1 || (ng / nfld) % kX) return cudaErrorInvalidValue;
-  const int imag = complex_out == 2 ? 1 : 0;  // real T holding Im(P a)
-  if (complex_out == 1) {
-    if (tcg == 4) return simt4_t<4, true>(astore, ng, delta, tiles, ntiles, rows, cols, uniq, nsplit, nsingle, T, nsm, imag, st, nfld, t_field_stride);
-    if (tcg == 8) return simt4_t<8, true>(astore, ng, delta, tiles, ntiles, rows, cols, uniq, nsplit, nsingle, T, nsm, imag, st, nfld, t_field_stride);
-    if (tcg == 16) return simt4_t<16, true>(astore, ng, delta, tiles, ntiles, rows, cols, uniq, nsplit, nsingle, T, nsm, imag, st, nfld, t_field_stride);
-  } else {
-    if (tcg == 4) return simt4_t<4, false>(astore, ng, delta, tiles, ntiles, rows, cols, uniq, nsplit, nsingle, T, nsm, imag, st, nfld, t_field_stride);
-    if (tcg == 8) return simt4_t<8, false>(astore, ng, delta, tiles, ntiles, rows, cols, uniq, nsplit, nsingle, T, nsm, imag, st, nfld, t_field_stride);
-    if (tcg == 16) return simt4_t<16, false>(astore, ng, delta, tiles, ntiles, rows, cols, uniq, nsplit, nsingle, T, nsm, imag, st, nfld, t_field_stride);
+SimtGeometry simt_geometry(int complex_t, int ncols) {
+  SimtGeometry g;
+  // 4 columns per thread where 8 would leave a quarter of them empty or more
+  // (128^3, lmax 4, 10 bins: 34.0 ms against 35.3 with 8 everywhere; 5 bins 4.5
+  // against 4.7)
+  const int c8 = (ncols + 7) / 8 * 8, c4 = (ncols + 3) / 4 * 4;
+  g.ct = complex_t || 4 * c4 <= 3 * c8 ? 4 : 8;
+  g.rt = complex_t ? 8 : 64 / g.ct;
+  g.ncg = (ncols + g.ct - 1) / g.ct;
+  // the most row groups that fill their warps well; at most 96 singles and
+  // simt_rows() rows keep a tile's shared memory near a quarter of an SM's
+  const int most = std::min(kSimtThreads / g.ncg, simt_rows(g.rt) / g.rt);
+  auto fill = [&](int n) { return n * g.ncg / (double)((n * g.ncg + 31) / 32 * 32); };
+  double best = 0.0;
+  for (int n = (most + 1) / 2; n <= most; ++n) best = std::max(best, fill(n));
+  int n = most;
+  while (fill(n) < best - 0.06) --n;
+  g.max_rows = g.rt * n;
+  g.max_uniq = 96;
+  return g;
+}
+
+long long simt_entry(const Tile4& t, const SimtGeometry& g, int r, int c) {
+  const int pr = r % (4 * t.nrg), pc = c % (4 * t.ncg);  // within the section
+  const int ri = r / (4 * t.nrg) * 4 + pr % 4, cj = c / (4 * t.ncg) * 4 + pc % 4;
+  const int i = ri / 2, e = ri & 1, j = cj / 2, w = (cj & 1) ^ e;
+  return t.tout + ((long long)((i * (g.ct / 2) + j) * 2 + w) * 2 + e) * (t.nrg * t.ncg) + pr / 4 * t.ncg + pc / 4;
+}
+
+size_t simt_tile_smem(const Tile4& t, const SimtGeometry& g) {
+  return simt_smem(simt_rows(g.rt), simt_cols(g.ct, g.rt * g.ct == 32), t.nuniq, t.ncols);
+}
+
+cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta, const Tile4* tiles,
+                         const SimtPlan& plan, const Row4* rows, const int* cols, const int* uniq, int complex_out,
+                         int nsingle, double* T, int nsm, cudaStream_t st, int* launches, int nfld,
+                         long long t_field_stride) {
+  if (ng % 32 || complex_out < 0 || complex_out > 2 || nfld < 1 || (ng / nfld) % 32) return cudaErrorInvalidValue;
+  SimtArgs a{};
+  a.astore = (const float*)astore;
+  a.delta = delta;
+  a.tiles = tiles;
+  a.rows = rows;
+  a.cols = cols;
+  a.uniq = uniq;
+  a.T = T;
+  a.ng = ng;
+  a.nsingle = nsingle;
+  a.imag = complex_out == 2 ? 1 : 0;  // real T holding Im(P a)
+  a.t_field_stride = t_field_stride;
+  // The x-splits of a column class: one field, as many as fill 2 .. 8 waves of
+  // the units (span_tiles x split) best on 2 (complex T: 1) units per SM; a slab,
+  // per field a power of two by the same measure.  They set where the FP32
+  // spans begin, hence the rounding of every result, and nothing else: the
+  // spans are dealt to CTAs in simt4_t, however many fit there.
+  const long long slots = (long long)nsm * (complex_out == 1 ? 1 : 2), chunks = ng / 32;
+  int spf[3] = {0, 0, 0};
+  for (int c = 0; c < 3; ++c) {
+    const long long nt = plan.span_tiles[c];
+    long long ns = 1;
+    double best = -1.0;
+    if (nt && nfld > 1) {
+      const long long fchunks = chunks / nfld;
+      spf[c] = 1;
+      for (long long k = 1; k <= fchunks && k <= 64; k *= 2) {
+        const long long units = nt * nfld * k;
+        if (units > 65535LL * nt) break;
+        const double fill = (double)units / (double)(slots * ((units + slots - 1) / slots));
+        if (fill > best + 1e-3) {
+          best = fill;
+          spf[c] = (int)k;
+        }
+        if (units >= 4 * slots) break;
+      }
+      ns = (long long)nfld * spf[c];
+    } else if (nt) {
+      for (int w = 2; w <= 8; ++w) {
+        const long long n = std::max<long long>(1, std::min<long long>(chunks, slots * w / nt));
+        const long long units = n * nt;
+        const double fill = (double)units / (double)(slots * ((units + slots - 1) / slots));
+        if (fill > best + 1e-3) {
+          best = fill;
+          ns = n;
+        }
+      }
+    }
+    SimtSpans& sp = a.sp[c];
+    sp.nsplit = (int)ns;
+    sp.per = (chunks + ns - 1) / ns * 32;
+    sp.nsp = (int)((sp.per + kSpan * kX - 1) / (kSpan * kX));
+    sp.unit = 1;
+    a.spf[c] = spf[c];
   }
-  return cudaErrorInvalidValue;
+  *launches = 0;
+  for (int k = 0; k < 2; ++k) {
+    if (!plan.ntiles[k]) continue;
+    cudaError_t e;
+    if (complex_out == 1) e = simt4_t<8, 4, true>(a, plan, k, nsm, st);
+    else if (k == 0) e = simt4_t<16, 4, false>(a, plan, k, nsm, st);
+    else e = simt4_t<8, 8, false>(a, plan, k, nsm, st);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+  }
+  return cudaSuccess;
 }
 
 // ------------------------------------------------------------- finalisation --

@@ -36,7 +36,8 @@ struct Tile4 {
   int col0, ncols;     // cols of the global col table
   int uniq0, nuniq;    // staged singles (store indices); tensor-core tiles: sorted slot list
   int bgroup;          // tensor-core tiles: the B image (column group) of the tile
-  int pad;
+  int cls;             // FP32 tiles: span class (0: <= 16 columns, 1: <= 32, 2: <= 64)
+  int nrg, ncg;        // FP32 tiles: row and column groups (threads) of the tile
   long long tout;      // offset (in outputs) of this tile's [nrows][ncols] block of T
 };
 struct Row4 {
@@ -45,14 +46,36 @@ struct Row4 {
   float sign;          // +-1 from a_{l,-m} = (-1)^m conj(a_{lm}) (3D)
 };
 
+// FP32 tiles of one plan, in two launches: [0] those of 4 columns per thread,
+// [1] those of 8.  The FP32 spans of a column class begin where x-splits chosen
+// for span_tiles units of 4096 entries (at most kSimtSpanUniq singles each) begin.
+constexpr int kSimtSpanUniq = 64;
+struct SimtPlan {
+  int span_tiles[3];
+  int first[2], ntiles[2];
+  int threads[2];      // the most thread positions (nrg ncg) of the launch's tiles
+  size_t smem[2];      // the most dynamic shared memory of its tiles
+  bool uses[2][3];     // the launch has tiles of the class
+};
+// FP32 tiles of ncols columns: rows and columns per thread, column groups, most
+// rows and most staged row singles.
+struct SimtGeometry {
+  int rt, ct, ncg, max_rows, max_uniq;
+};
+SimtGeometry simt_geometry(int complex_t, int ncols);
+// Index in T of entry (row r, column c) of an FP32 tile, which occupies
+// [tout, tout + rt ct nrg ncg).
+long long simt_entry(const Tile4& t, const SimtGeometry& g, int r, int c);
+size_t simt_tile_smem(const Tile4& t, const SimtGeometry& g);
+
 // T[tile][r][c] (+)= sum_x delta * f1 * f2 * a_col: its real part
 // (complex_out 0), complex value (1, two doubles per entry) or imaginary part
-// (2).  nsplit <= 0: x-splits per tile chosen to fill whole waves of nsm SMs.
+// (2).  *launches receives the kernels launched.
 // A slab of nfld fields (ng = nfld x the points of one field): each field is
 // split alike and adds into T + f t_field_stride (doubles).
 cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta, const Tile4* tiles,
-                         int ntiles, const Row4* rows, const int* cols, const int* uniq, int complex_out,
-                         int tcg, int nsplit, int nsingle, double* T, int nsm, cudaStream_t st, int nfld = 1,
+                         const SimtPlan& plan, const Row4* rows, const int* cols, const int* uniq, int complex_out,
+                         int nsingle, double* T, int nsm, cudaStream_t st, int* launches, int nfld = 1,
                          long long t_field_stride = 0);
 
 // Tensor-core (tcgen05) split-BF16 version of the same contraction (sbg_tc.cu).
@@ -69,7 +92,6 @@ cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta,
 // withholds the kernel's MMA issuer, so that the other roles' waits run out (a
 // host-side test of the timeout path; nothing is computed).
 constexpr int kTcMaxRowSlots = 56;  // row singles staged per K-block
-constexpr int kSimtMaxUniq = 64;    // row singles staged per chunk by the FP32 SIMT kernel
 constexpr int kTcEpoch = 256;       // K-blocks between progress checkpoints of the lag limiter
 struct BGroup {
   int col0, ncols;     // columns (global col table)
