@@ -190,6 +190,7 @@ struct sbg_context {
   };
   bool defer = false;
   int cur = 0;
+  std::string xf_key;  // what the transform table in buffer "xf" was made for
   // autotuner: launch choices measured on their first use, by key
   std::map<std::string, int> tune;
   cudaEvent_t tev[2] = {};
@@ -1074,14 +1075,13 @@ sbg_status tune_fft(sbg_context* ctx, int n, FftPass& p) {
   q.nb_per_field = 0;
   q.shared_stride = 0;
   q.field_points = 0;
-  if (q.npack) q.npack = std::min(q.npack, 2 * q.batch);
   void* scratch;
   ST(buf(ctx, "tune", (size_t)q.batch * (size_t)q.bstride * 8, &scratch));
   q.out = (float2*)scratch;
   std::vector<int> cands = {0, 1};
   // twice the lines: up to N = 512, and N = 256 for the product passes (which
   // also stage delta-hat in shared memory)
-  const bool product = p.load == LOAD_MUL || p.load == LOAD_MUL2;
+  const bool product = p.load == LOAD_MUL || p.load == LOAD_MUL2 || p.load == LOAD_MULT;
   if (n <= (product ? 256 : 512)) cands.push_back(2);
   int tl = 0;
   ST(autotune(ctx, key, cands, [&](int c) { q.tl = c; return fft_axis_pass(n, q, ctx->stream); }, &tl));
@@ -1090,87 +1090,159 @@ sbg_status tune_fft(sbg_context* ctx, int n, FftPass& p) {
 }
 
 // -------------------------------------------------------- FFT helpers ----
-// 3D transform in three axis passes; with final_out the last pass writes the
-// blocked coefficient store (singles single0 .. single0 + batch - 1 of nsingle).
-// npack > 0 (with LOAD_MUL and final_out): the npack factor arrays give
-// transforms with real results, packed two per complex transform (LOAD_MUL2,
-// batch = (npack + 1) / 2) and written back as singles single0 .. + npack - 1.
-sbg_status fft3(sbg_context* ctx, int n, int sign, int first_load, const void* in, float2* out, const float2* mul,
-                const float2* shared, int batch, const float2* tw, float2* final_out = nullptr, int nsingle = 0,
-                int single0 = 0, int prune_r = -1, int npack = 0) {
-  const long long ng = (long long)n * n * n;
+// Transform of `batch` arrays in three (dim 3) or two axis passes, in place in
+// `out` after the first.  prune_r >= 0 (dim 3): the input is zero beyond
+// minimum-image distance prune_r on every axis, so z-lines outside the (y, x)
+// support and, after that pass, y-lines outside the x support stay zero and are
+// skipped.
+sbg_status fft_all(sbg_context* ctx, int dim, int n, int sign, int load, const void* in, float2* out, int batch,
+                   const float2* tw, int prune_r = -1) {
   FftPass p{};
   p.twiddle = tw;
   p.batch = batch;
-  p.bstride = ng;
+  p.bstride = dim == 3 ? (long long)n * n * n : (long long)n * n;
   p.sign = sign;
-  if (npack > 0) {
-    if (first_load != LOAD_MUL || !final_out || batch != (npack + 1) / 2) return fail(ctx, SBG_ERR_INTERNAL, "fft3 packing");
-    first_load = LOAD_MUL2;
-    p.npack = npack;
+  p.in = in; p.out = out; p.load = load;
+  if (dim == 3) {  // z axis
+    p.outer = 1; p.inner = (long long)n * n;
+    if (prune_r >= 0) { p.prune_mode = 1; p.prune_r = prune_r; }
+    ST(tune_fft(ctx, n, p));
+    KL(fft_axis_pass(n, p, ctx->stream));
+    p.tl = 0;
+    p.in = out; p.load = LOAD_COMPLEX;
   }
-  // z axis (strided by n^2), fused first-pass load
-  p.in = in; p.out = out; p.mul = mul; p.shared = shared; p.load = first_load;
-  p.outer = 1; p.inner = (long long)n * n;
-  // prune_r >= 0: the input is zero beyond minimum-image distance prune_r on
-  // every axis, so z-lines outside the (y, x) support and, after that pass,
-  // y-lines outside the x support stay zero and are skipped
-  if (prune_r >= 0) { p.prune_mode = 1; p.prune_r = prune_r; }
-  ST(tune_fft(ctx, n, p));
-  KL(fft_axis_pass(n, p, ctx->stream));
-  // y axis
-  p.in = out; p.load = LOAD_COMPLEX; p.mul = nullptr; p.shared = nullptr;
-  p.outer = n; p.inner = n;
+  p.outer = dim == 3 ? n : 1; p.inner = n;  // y axis
   if (prune_r >= 0) p.prune_mode = 2;
-  p.tl = 0;
   ST(tune_fft(ctx, n, p));
   KL(fft_axis_pass(n, p, ctx->stream));
   p.tl = 0;
-  // x axis (contiguous)
   p.prune_mode = 0;
-  p.outer = (long long)n * n; p.inner = 1;
-  if (final_out) {
-    p.out = final_out; p.out_blocked = npack > 0 ? 2 : 1; p.nsingle = nsingle; p.single0 = single0;
-  }
+  p.in = out; p.load = LOAD_COMPLEX;
+  p.outer = dim == 3 ? (long long)n * n : n; p.inner = 1;  // x axis
   KL(fft_axis_pass(n, p, ctx->stream));
   return SBG_OK;
 }
 
-// nfld > 1: a slab of fields, batch = nfld x arrays per field; `shared` is per
-// field (stride shared_stride) and the blocked store's points of field f start
-// at f x bstride.
-sbg_status fft2(sbg_context* ctx, int n, int sign, int first_load, const void* in, float2* out, const float2* mul,
-                const float2* shared, int batch, long long bstride, const float2* tw, float2* final_out = nullptr,
-                int nsingle = 0, int single0 = 0, int npack = 0, int nfld = 1, long long shared_stride = 0) {
+// The inverse transforms of the convolutions: those of the stored groups
+// (g < ngroups4) go to the blocked coefficient store, where an m = 0 group (real
+// kernels, so real coefficients) takes two bins per transform; the other groups
+// take one transform per bin.  By group, or (pairs_first) the stored groups'
+// packed transforms before their others, so that one launch of each kind serves
+// every group.
+struct ConvTable {
+  std::vector<FftXf> xf;
+  std::vector<int> first;  // by group: first transform of each group, and the count
+  std::vector<char> real;  // by group: its transforms are packed real ones
+  int stored = 0;          // transforms of stored groups
+  int packed = 0;          // packed ones
+};
+ConvTable conv_table(int dim, int nb, int ngroups, int ngroups4, bool pairs_first) {
+  ConvTable t;
+  std::vector<FftXf> single;
+  for (int g = 0, l = 0; g < ngroups; ++g) {
+    if (g == ngroups4) t.xf.insert(t.xf.end(), single.begin(), single.end());
+    t.first.push_back((int)t.xf.size());
+    while (dim == 3 && (l + 1) * (l + 2) / 2 <= g) ++l;
+    const bool m0 = dim == 3 ? g == l * (l + 1) / 2 : g == 0;
+    t.real.push_back(m0 && g < ngroups4);
+    if (t.real[g]) {
+      for (int b = 0; b < nb; b += 2) t.xf.push_back({g * nb + b, b + 1 < nb ? g * nb + b + 1 : -1, g * nb + b, 0});
+      t.packed += (nb + 1) / 2;
+    } else {
+      auto& to = pairs_first && g < ngroups4 ? single : t.xf;
+      for (int b = 0; b < nb; ++b) to.push_back({g * nb + b, -1, g * nb + b, 0});
+    }
+    if (g < ngroups4) t.stored += m0 ? (nb + 1) / 2 : nb;
+  }
+  if (ngroups <= ngroups4) t.xf.insert(t.xf.end(), single.begin(), single.end());
+  t.first.push_back((int)t.xf.size());
+  return t;
+}
+
+// Groups whose convolutions one launch of each pass takes: as many as keep the
+// arrays between the passes (`bytes` each, for all fields of a slab) within
+// kConvBytes, so that small grids take few launches, and at least one.  Measured
+// (convolutions and Gram): 64^2, 20 transforms, 85 -> 18 us and 256^2, 55
+// transforms, 216 -> 60 us against one group per launch; beyond that size more
+// transforms per launch gain nothing (256^3, 10 of two arrays instead of 5: 80
+// instead of 73 us each), and fewer than a group's, to keep the arrays in L2,
+// lose (1024^2, 20 bins: 1.54 ms by groups, 1.88 ms by 32 MB).
+constexpr long long kConvBytes = 48 << 20;
+int conv_groups(int nb, long long bytes) { return (int)std::max<long long>(1, kConvBytes / (bytes * nb)); }
+
+// Convolutions a = IFFT(delta-hat G) of the transforms [t0, t1) of the table d_xf
+// (device) in one launch per pass: product and z (dim 3) or y pass, y pass (dim
+// 3), x pass.  `load` says how the product takes its factors; G holds the factor
+// arrays from array a0 on (LOAD_MUL: those of t0 ...).  astore != null: the x pass
+// writes the blocked store of nsingle singles, through `work`; else the
+// transforms go to work, [field][transform].
+sbg_status conv_run(sbg_context* ctx, int dim, int n, const FftXf* d_xf, int t0, int t1, int load, const float2* G,
+                    int a0, const float2* dhat, const float2* tw, float2* work, float2* astore, int nsingle,
+                    int nfld = 1) {
+  if (t0 >= t1) return SBG_OK;
+  const long long ng = dim == 3 ? (long long)n * n * n : (long long)n * n;
   FftPass p{};
   p.twiddle = tw;
-  p.batch = batch;
-  p.bstride = bstride;
-  p.sign = sign;
+  p.batch = nfld * (t1 - t0);
+  p.bstride = ng;
+  p.sign = +1;
+  p.xf = d_xf + t0;
+  p.a0 = a0;
   if (nfld > 1) {
-    if (batch % nfld) return fail(ctx, SBG_ERR_INTERNAL, "fft2 slab batch");
-    p.nb_per_field = batch / nfld;
-    p.shared_stride = shared_stride;
-    p.field_points = bstride;
+    p.nb_per_field = t1 - t0;
+    p.shared_stride = ng;
+    p.field_points = ng;
   }
-  if (npack > 0) {  // as in fft3
-    if (first_load != LOAD_MUL || !final_out || batch != nfld * ((npack + 1) / 2))
-      return fail(ctx, SBG_ERR_INTERNAL, "fft2 packing");
-    first_load = LOAD_MUL2;
-    p.npack = npack;
-  }
-  p.in = in; p.out = out; p.mul = mul; p.shared = shared; p.load = first_load;
-  p.outer = 1; p.inner = n;  // y axis
+  p.out = work; p.mul = G; p.shared = dhat; p.load = load;
+  p.outer = 1; p.inner = ng / n;
   ST(tune_fft(ctx, n, p));
   KL(fft_axis_pass(n, p, ctx->stream));
   p.tl = 0;
-  p.in = out; p.load = LOAD_COMPLEX; p.mul = nullptr; p.shared = nullptr;
-  p.outer = n; p.inner = 1;  // x axis
-  if (final_out) {
-    p.out = final_out; p.out_blocked = npack > 0 ? 2 : 1; p.nsingle = nsingle; p.single0 = single0;
+  p.in = work; p.load = LOAD_COMPLEX; p.mul = nullptr; p.shared = nullptr;
+  if (dim == 3) {
+    p.outer = n; p.inner = n;
+    ST(tune_fft(ctx, n, p));
+    KL(fft_axis_pass(n, p, ctx->stream));
+    p.tl = 0;
   }
+  p.outer = ng / n; p.inner = 1;
+  if (astore) { p.out = astore; p.out_blocked = load == LOAD_MUL2 ? 2 : 1; p.nsingle = nsingle; }
   KL(fft_axis_pass(n, p, ctx->stream));
   return SBG_OK;
+}
+
+// Every stored group's convolutions, at most `most` transforms of one kind per
+// launch (table in pairs_first order).
+sbg_status conv_stored(sbg_context* ctx, int dim, int n, const FftXf* d_xf, const ConvTable& t, int most, const float2* G,
+                       const float2* dhat, const float2* tw, float2* work, float2* astore, int nsingle, int nfld = 1) {
+  for (int i = 0, c; i < t.stored; i += c) {
+    const bool packed = i < t.packed;
+    c = std::min(most, (packed ? t.packed : t.stored) - i);
+    ST(conv_run(ctx, dim, n, d_xf, i, i + c, packed ? LOAD_MUL2 : LOAD_MULT, G, 0, dhat, tw, work, astore, nsingle, nfld));
+  }
+  return SBG_OK;
+}
+
+// The table of this call's transforms on the device (kept while it stays the same).
+sbg_status conv_upload(sbg_context* ctx, const ConvTable& t, int dim, int nb, int ngroups, int ngroups4, bool pairs_first,
+                       FftXf** out) {
+  ST(buf(ctx, "xf", t.xf.size() * sizeof(FftXf), (void**)out));
+  const std::string key = std::to_string(dim) + "/" + std::to_string(nb) + "/" + std::to_string(ngroups) + "/" +
+                          std::to_string(ngroups4) + (pairs_first ? "/p" : "");
+  if (ctx->xf_key != key) {
+    ctx->xf_key.clear();
+    CU(cudaMemcpyAsync(*out, t.xf.data(), t.xf.size() * sizeof(FftXf), cudaMemcpyHostToDevice, ctx->stream));
+    ctx->xf_key = key;
+  }
+  return SBG_OK;
+}
+
+// Groups per launch of a call's convolutions (see conv_groups) and the buffer
+// "group" that holds their arrays.  A context with a budget takes one (its other
+// buffers have to fit as well).
+sbg_status conv_buffer(sbg_context* ctx, int nb, int ngroups, long long bytes, int* per, float2** out) {
+  *per = ctx->budget ? 1 : std::min(ngroups, conv_groups(nb, bytes));
+  return buf(ctx, "group", (size_t)*per * nb * bytes, (void**)out);
 }
 
 sbg_status check_edges(sbg_context* ctx, const double* edges, int nb, int n) {
@@ -1272,11 +1344,7 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
   KL(launch_convert(d_in, dtype == SBG_F64, ng, d_acc, (flags & SBG_SUBTRACT_MEAN) ? 1 : 0, d_delta, ctx->stream));
   rec(ctx, 1);
   // ---- delta-hat ----
-  if (dim == 3) {
-    ST(fft3(ctx, n, -1, LOAD_REAL, d_delta, d_dhat, nullptr, nullptr, 1, d_tw));
-  } else {
-    ST(fft2(ctx, n, -1, LOAD_REAL, d_delta, d_dhat, nullptr, nullptr, 1, ng, d_tw));
-  }
+  ST(fft_all(ctx, dim, n, -1, LOAD_REAL, d_delta, d_dhat, 1, d_tw));
   rec(ctx, 2);
   // ---- kernel spectra (plan) ----
   char keyb[512];
@@ -1286,18 +1354,18 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
   const size_t gbytes = (size_t)ngroups * nb * ng * 8;
   const double inv_ng = 1.0 / (double)ng;
   auto gen_group = [&](int g, float2* dst) -> sbg_status {
-    CU(cudaMemsetAsync(dst, 0, (size_t)nb * ng * 8, ctx->stream));
     if (dim == 3) {
+      CU(cudaMemsetAsync(dst, 0, (size_t)nb * ng * 8, ctx->stream));
       int l = 0;
       while ((l + 1) * (l + 2) / 2 <= g) ++l;
       const int m = g - l * (l + 1) / 2;
       KL(launch_kgen3d(n, l, m, ylm_norm(l, m), d_e2, nb, inv_ng, dst, ctx->stream));
       // the kernels vanish beyond the last edge: prune the zero lines
       const int rmax = std::min(n / 2 - 1, (int)std::ceil(edges[nb]));
-      ST(fft3(ctx, n, +1, LOAD_COMPLEX, dst, dst, nullptr, nullptr, nb, d_tw, nullptr, 0, 0, rmax));
+      ST(fft_all(ctx, 3, n, +1, LOAD_COMPLEX, dst, dst, nb, d_tw, rmax));
     } else {
-      KL(launch_kgen2d(n, g, d_e2, nb, inv_ng, dst, ctx->stream));
-      ST(fft2(ctx, n, +1, LOAD_COMPLEX, dst, dst, nullptr, nullptr, nb, ng, d_tw));
+      KL(launch_kgen2d(n, g, 1, d_e2, nb, inv_ng, dst, ctx->stream));
+      ST(fft_all(ctx, 2, n, +1, LOAD_COMPLEX, dst, dst, nb, d_tw));
     }
     return SBG_OK;
   };
@@ -1329,7 +1397,15 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
   double* d_S = nullptr;
   const int nsingle = ngroups4 * nb;  // singles in the blocked coefficient store
   if (do4) ST(buf(ctx, "astore", (size_t)nsingle * ng * 8, (void**)&d_astore));
-  ST(buf(ctx, "group", (size_t)nb * ng * 8, (void**)&d_group));
+  const bool fused = dim == 3 && !cached;  // see below
+  int per = 1;  // groups per launch
+  ST(conv_buffer(ctx, nb, ngroups, ng * 8, &per, &d_group));
+  if (!cached) per = 1;
+  // the stored groups' transforms by kind when several groups fit
+  const bool together = per > 1 && ngroups4 > 0;
+  const ConvTable conv = conv_table(dim, nb, ngroups, ngroups4, together);
+  FftXf* d_xf = nullptr;
+  ST(conv_upload(ctx, conv, dim, nb, ngroups, ngroups4, together, &d_xf));
   float2* d_gtmp = nullptr;
   if (!cached) ST(buf(ctx, "gtmp", (size_t)nb * ng * 8, (void**)&d_gtmp));
   const int ngroups3 = do3 ? npair(lmax3) : 0;
@@ -1351,7 +1427,6 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
   // FFT and the spectral product fused between the forward and inverse z
   // transforms (sbg_fft_fused.cu); the lines of the kernel support are listed
   // once per call
-  const bool fused = dim == 3 && !cached;
   int* d_lines = nullptr;
   int nlines = 0, Rsup = 0;
   if (fused) {
@@ -1366,30 +1441,27 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
     ST(buf(ctx, "klines", std::max<size_t>(lines.size(), 1) * 4, (void**)&d_lines));
     if (nlines) CU(cudaMemcpyAsync(d_lines, lines.data(), lines.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
   }
-  int gpend = -1;  // a stored group whose Gram waits for the next one's
-  for (int g = 0; g < ngroups; ++g) {
-    const float2* G = nullptr;
-    if (cached) {
-      G = (const float2*)ctx->gcache.p + (size_t)g * nb * ng;
-    } else if (!fused) {
-      ST(gen_group(g, d_gtmp));
-      G = d_gtmp;
-    }
-    const bool stored = g < ngroups4;
-    float2* fin = stored ? d_astore : nullptr;
-    // m = 0: the kernels are real (Y_l0 is real; e^{-i 0 phi} = 1), so with a
-    // real delta every a^b is real and two bins share one complex inverse
-    // transform; only for stored groups (the 3PCF Gram of the others reads the
-    // transform output directly)
-    int l0 = 0;
-    while (dim == 3 && (l0 + 1) * (l0 + 2) / 2 <= g) ++l0;
-    const bool m0 = dim == 3 ? g == l0 * (l0 + 1) / 2 : g == 0;
-    const int npack = stored && m0 ? nb : 0;
-    const int nbatch = npack ? (nb + 1) / 2 : nb;
-    if (fused) {
-      int l = 0;
+  // delta-weighted Grams of the groups [g0, g1) in one launch: from the blocked
+  // store, or from the group buffer
+  auto gram = [&](int g0, int g1, bool stored) -> sbg_status {
+    g1 = std::min(g1, ngroups3);
+    if (!do3 || g0 >= g1) return SBG_OK;
+    double* Sg = d_S + (size_t)g0 * nb * nb * 2;
+    const float2* src = stored ? d_astore : d_group;
+    const int ns = stored ? nsingle : 0, s0 = stored ? g0 * nb : 0;
+    if (tcomb)
+      KL(launch_gram_tc(src, ng, nb, d_delta, Sg, ns, s0, tf32, d_err, ctx->nsm, ctx->wait_ns, ctx->stall, ctx->stream, 1,
+                        0, g1 - g0));
+    else
+      KL(launch_gram3(src, ng, nb, d_delta, Sg, ns, s0, ctx->stream, 1, 0, g1 - g0));
+    return SBG_OK;
+  };
+  if (fused) {
+    for (int g = 0, l = 0; g < ngroups; ++g) {
       while ((l + 1) * (l + 2) / 2 <= g) ++l;
       const int m = g - l * (l + 1) / 2;
+      const bool stored = g < ngroups4;
+      const int nbatch = conv.first[g + 1] - conv.first[g];
       FusedGroup fg{};
       fg.l = l;
       fg.m = m;
@@ -1400,7 +1472,7 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
       fg.lines = d_lines;
       fg.nlines = nlines;
       fg.R = Rsup;
-      fg.npack = npack;
+      fg.npack = stored && m == 0 ? nb : 0;
       fg.tw = d_tw;
       fg.kbuf = d_gtmp;
       fg.dhat = d_dhat;
@@ -1423,37 +1495,37 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
       p.tl = 0;
       p.outer = (long long)n * n;
       p.inner = 1;
-      if (fin) {
-        p.out = fin;
-        p.out_blocked = npack > 0 ? 2 : 1;
+      if (stored) {
+        p.out = d_astore;
+        p.out_blocked = m == 0 ? 2 : 1;
         p.nsingle = nsingle;
-        p.single0 = g * nb;
-        p.npack = npack;
+        p.xf = d_xf + conv.first[g];
       }
       KL(fft_axis_pass(n, p, ctx->stream));
-    } else if (dim == 3) {
-      ST(fft3(ctx, n, +1, LOAD_MUL, nullptr, d_group, G, d_dhat, nbatch, d_tw, fin, nsingle, g * nb, -1, npack));
-    } else {
-      ST(fft2(ctx, n, +1, LOAD_MUL, nullptr, d_group, G, d_dhat, nbatch, ng, d_tw, fin, nsingle, g * nb, npack));
+      if (!stored) ST(gram(g, g + 1, false));
     }
-    if (do3 && g < ngroups3) {
-      // two adjacent stored groups are one launch of the tensor-core Gram
-      // (their singles sit side by side in the blocked store)
-      const bool pair = tcomb && stored && 2 * nb <= kGramTcMaxNb;
-      if (pair && gpend < 0 && g + 1 < std::min(ngroups3, ngroups4)) {
-        gpend = g;
-      } else {
-        const int g0 = gpend >= 0 ? gpend : g, k = g - g0 + 1;
-        gpend = -1;
-        double* Sg = d_S + (size_t)g0 * nb * nb * 2;
-        const float2* src = stored ? d_astore : d_group;
-        const int ns = stored ? nsingle : 0, s0 = stored ? g0 * nb : 0;
-        if (tcomb) KL(launch_gram_tc(src, ng, k * nb, d_delta, Sg, ns, s0, tf32, d_err, ctx->nsm, ctx->wait_ns,
-                                     ctx->stall, ctx->stream, 1, 0, k, (long long)nb * nb * 2));
-        else KL(launch_gram3(src, ng, nb, d_delta, Sg, ns, s0, ctx->stream));
-      }
+  } else {
+    const float2* G = cached ? (const float2*)ctx->gcache.p : d_gtmp;
+    int g0 = 0;
+    if (together) {
+      ST(conv_stored(ctx, dim, n, d_xf, conv, per * nb, G, d_dhat, d_tw, d_group, d_astore, nsingle));
+      g0 = ngroups4;
+    }
+    // the others in order: several 2D groups per launch where the spectra are
+    // cached, else one by one (3D: step by step like the fused path)
+    for (int g1; g0 < ngroups; g0 = g1) {
+      const bool stored = g0 < ngroups4;
+      g1 = dim == 2 && !stored ? std::min(ngroups, g0 + per) : g0 + 1;
+      const int t0 = conv.first[g0], t1 = conv.first[g1];
+      const bool pairs = conv.real[g0];
+      if (!cached) ST(gen_group(g0, d_gtmp));
+      ST(conv_run(ctx, dim, n, d_xf, t0, t1, pairs ? LOAD_MUL2 : LOAD_MUL,
+                  cached && !pairs ? G + (long long)g0 * nb * ng : G, cached ? 0 : g0 * nb, d_dhat, d_tw, d_group,
+                  stored ? d_astore : nullptr, nsingle));
+      if (!stored) ST(gram(g0, g1, false));
     }
   }
+  ST(gram(0, ngroups4, true));
   rec(ctx, 4);
   rec(ctx, 5);
   // ---- 4PCF ----
@@ -1655,7 +1727,7 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
   KL(launch_convert(d_in, dtype == SBG_F64, ng, d_acc, (flags & SBG_SUBTRACT_MEAN) ? 1 : 0, d_delta, st, nfld));
   rec(ctx, 1);
   // ---- delta-hat of every field ----
-  ST(fft2(ctx, n, -1, LOAD_REAL, d_delta, d_dhat, nullptr, nullptr, nfld, ng, d_tw));
+  ST(fft_all(ctx, 2, n, -1, LOAD_REAL, d_delta, d_dhat, nfld, d_tw));
   rec(ctx, 2);
   // ---- kernel spectra (shared by the fields: one shape, one bin set) ----
   char keyb[512];
@@ -1665,9 +1737,8 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
   const size_t gbytes = (size_t)ngroups * nb * ng * 8;
   const double inv_ng = 1.0 / (double)ng;
   auto gen_group = [&](int g, float2* dst) -> sbg_status {
-    CU(cudaMemsetAsync(dst, 0, (size_t)nb * ng * 8, st));
-    KL(launch_kgen2d(n, g, d_e2, nb, inv_ng, dst, st));
-    ST(fft2(ctx, n, +1, LOAD_COMPLEX, dst, dst, nullptr, nullptr, nb, ng, d_tw));
+    KL(launch_kgen2d(n, g, 1, d_e2, nb, inv_ng, dst, st));
+    ST(fft_all(ctx, 2, n, +1, LOAD_COMPLEX, dst, dst, nb, d_tw));
     return SBG_OK;
   };
   const float2* gbase = nullptr;
@@ -1709,7 +1780,13 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
   float2* d_astore = nullptr;
   if (do4) ST(buf(ctx, "astore", (size_t)nsingle * npts * 8, (void**)&d_astore));
   float2* d_group;
-  ST(buf(ctx, "group", (size_t)nfld * nb * ng * 8, (void**)&d_group));
+  int per = 1;  // groups per launch
+  ST(conv_buffer(ctx, nb, std::max(1, std::min(ngroups, 65535 / (nfld * nb))), nfld * ng * 8, &per, &d_group));
+  if (!cached) per = 1;
+  const bool together = do4 && per > 1;  // as in measure()
+  const ConvTable conv = conv_table(2, nb, ngroups, ngroups4, together);
+  FftXf* d_xf = nullptr;
+  ST(conv_upload(ctx, conv, 2, nb, ngroups, ngroups4, together, &d_xf));
   float2* d_gtmp = nullptr;
   if (!cached) ST(buf(ctx, "gtmp", (size_t)nb * ng * 8, (void**)&d_gtmp));
   const int ngroups3 = do3 ? mmax + 1 : 0;
@@ -1723,40 +1800,36 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
   const int tf32 = prec == SBG_PREC_TF32X3 ? 1 : 0;
   int* d_err = nullptr;
   if (tcomb) ST(buf(ctx, "err", 16, (void**)&d_err));  // cleared by the caller once per batch
-  int gpend = -1;  // a stored group whose Gram waits for the next one's
-  for (int g = 0; g < ngroups; ++g) {
-    const float2* G;
-    if (cached) {
-      G = (const float2*)gbase + (size_t)g * nb * ng;
-    } else {
-      ST(gen_group(g, d_gtmp));
-      G = d_gtmp;
-    }
-    const bool stored = g < ngroups4;
-    float2* fin = stored ? d_astore : nullptr;
-    const int npack = stored && g == 0 ? nb : 0;  // m = 0: real coefficients, two bins per transform
-    const int nbatch = npack ? (nb + 1) / 2 : nb;
-    ST(fft2(ctx, n, +1, LOAD_MUL, nullptr, d_group, G, d_dhat, nfld * nbatch, ng, d_tw, fin, nsingle, g * nb, npack,
-            nfld, ng));
-    if (do3 && g < ngroups3) {
-      // two adjacent stored groups are one launch of the tensor-core Gram
-      const bool pair = tcomb && stored && 2 * nb <= kGramTcMaxNb;
-      if (pair && gpend < 0 && g + 1 < std::min(ngroups3, ngroups4)) {
-        gpend = g;
-      } else {
-        const int g0 = gpend >= 0 ? gpend : g, k = g - g0 + 1;
-        gpend = -1;
-        double* Sg = d_S + (size_t)g0 * nb * nb * 2;
-        const float2* src = stored ? d_astore : d_group;
-        const int ns = stored ? nsingle : 0, s0 = stored ? g0 * nb : 0;
-        if (tcomb)
-          KL(launch_gram_tc(src, ng, k * nb, d_delta, Sg, ns, s0, tf32, d_err, ctx->nsm, ctx->wait_ns, ctx->stall, st,
-                            nfld, s_stride, k, (long long)nb * nb * 2));
-        else
-          KL(launch_gram3(src, ng, nb, d_delta, Sg, ns, s0, st, nfld, s_stride));
-      }
-    }
+  // (every group is stored, or none)
+  auto gram = [&](int g0, int g1, bool stored) -> sbg_status {
+    if (!do3 || g0 >= g1) return SBG_OK;
+    double* Sg = d_S + (size_t)g0 * nb * nb * 2;
+    const float2* src = stored ? d_astore : d_group;
+    const int ns = stored ? nsingle : 0, s0 = stored ? g0 * nb : 0;
+    if (tcomb)
+      KL(launch_gram_tc(src, ng, nb, d_delta, Sg, ns, s0, tf32, d_err, ctx->nsm, ctx->wait_ns, ctx->stall, st, nfld,
+                        s_stride, g1 - g0));
+    else
+      KL(launch_gram3(src, ng, nb, d_delta, Sg, ns, s0, st, nfld, s_stride, g1 - g0));
+    return SBG_OK;
+  };
+  const float2* G = cached ? gbase : d_gtmp;
+  int g0 = 0;
+  if (together) {
+    ST(conv_stored(ctx, 2, n, d_xf, conv, per * nb, G, d_dhat, d_tw, d_group, d_astore, nsingle, nfld));
+    g0 = ngroups;
   }
+  for (int g1; g0 < ngroups; g0 = g1) {
+    g1 = do4 ? g0 + 1 : std::min(ngroups, g0 + per);
+    const int t0 = conv.first[g0], t1 = conv.first[g1];
+    const bool pairs = conv.real[g0];
+    if (!cached) ST(gen_group(g0, d_gtmp));
+    ST(conv_run(ctx, 2, n, d_xf, t0, t1, pairs ? LOAD_MUL2 : LOAD_MUL,
+                cached && !pairs ? G + (long long)g0 * nb * ng : G, cached ? 0 : g0 * nb, d_dhat, d_tw, d_group, d_astore,
+                nsingle, nfld));
+    if (!do4) ST(gram(g0, g1, false));
+  }
+  if (do4) ST(gram(0, ngroups, true));
   rec(ctx, 4);
   rec(ctx, 5);
   // ---- 4PCF of every field ----

@@ -17,33 +17,42 @@ __host__ __device__ __forceinline__ float2 csub(float2 a, float2 b) { return mak
 __host__ __device__ __forceinline__ float2 cconj(float2 a) { return make_float2(a.x, -a.y); }
 
 // Launch-time knobs shared by the FFT launchers.
-// LOAD_MUL2: batch j multiplies `shared` by mul_{2j} + i mul_{2j+1} (mul_{2j+1}
-// taken as 0 past npack arrays), so that two transforms with real results share
-// one complex transform
-enum FftLoad { LOAD_COMPLEX = 0, LOAD_REAL = 1, LOAD_MUL = 2, LOAD_MUL2 = 3 };
+// LOAD_MUL: `shared` times factor array j for transform j; LOAD_MULT: times the
+// factor array that the table names; LOAD_MUL2: times a + i b of the table.  (The
+// table's indirection costs the large product passes: 512^3, cached spectra, 6%
+// of the call.)
+enum FftLoad { LOAD_COMPLEX = 0, LOAD_REAL = 1, LOAD_MUL = 2, LOAD_MUL2 = 3, LOAD_MULT = 4 };
+
+// One inverse transform of the convolutions: its factor is array a, or
+// a + i b when b >= 0 (two transforms with real results share one complex
+// transform).  In the blocked coefficient store it is single s, and a packed
+// one's imaginary part single s + 1 (b >= 0).
+struct FftXf {
+  int a, b, s, pad;
+};
 
 // One axis pass of a batched 3D/2D complex FFT.  The array is viewed as
 // [batch][outer][N][inner]; the pass transforms along the N axis.
 struct FftPass {
   const void* in;        // float2 (or float for LOAD_REAL) base of batch 0
   float2* out;           // base of batch 0 (may alias `in`)
-  const float2* mul;     // LOAD_MUL: per-batch factor array (batch stride = bstride)
-  const float2* shared;  // LOAD_MUL: array common to every batch (e.g. delta-hat)
+  const float2* mul;     // LOAD_MUL*: factor arrays, bstride apart
+  const float2* shared;  // LOAD_MUL*: array common to every batch (e.g. delta-hat)
   const float2* twiddle; // N-entry table exp(sign 2 pi i j / N)
   long long outer, inner;
   long long bstride;     // elements between batches (in, out and mul)
   int batch;
   int sign;              // -1 forward, +1 inverse (unnormalised)
   int load;              // FftLoad
-  // Contiguous (last) pass only: with out_blocked = 1, batch b of the output
-  // goes to the blocked coefficient store as single s = single0 + b (see
-  // blocked_re); with out_blocked = 2 (the packed batches of LOAD_MUL2), the
-  // real part of batch b goes to single0 + 2b and the imaginary part to
-  // single0 + 2b + 1 (if 2b + 1 < npack), each with imaginary part 0.
+  // LOAD_MULT, LOAD_MUL2 and blocked output: the batch's transforms; factor
+  // array 0 of `mul` is array a0 of the table
+  const FftXf* xf;
+  int a0;
+  // Contiguous (last) pass only: the output goes to the blocked coefficient
+  // store of nsingle singles (see blocked_re), as `xf` says; out_blocked = 1:
+  // complex results, 2: packed real ones, stored with imaginary part 0.
   int out_blocked;
-  int npack;
   int nsingle;
-  int single0;
   // Strided passes only: skip line groups that are known to be all zero (a
   // kernel whose support lies within minimum-image distance prune_r of the
   // origin on every axis; the skipped lines must already hold zeros).
@@ -51,11 +60,10 @@ struct FftPass {
   //   prune_mode 2: inner index = x (second pass).
   int prune_mode;
   int prune_r;
-  // A slab of fields (0: one field): batch b is array b % nb_per_field of
-  // field b / nb_per_field; the factor array of LOAD_MUL / LOAD_MUL2 is taken
-  // per array of a field (offset (b % nb_per_field) bstride), `shared` per
-  // field (offset (b / nb_per_field) shared_stride), and a blocked-store
-  // output puts field f's points at f field_points onwards.
+  // A slab of fields (0: one field): batch b is transform b % nb_per_field of
+  // field b / nb_per_field; `shared` is taken per field (offset
+  // (b / nb_per_field) shared_stride), and a blocked-store output puts field
+  // f's points at f field_points onwards.
   int nb_per_field;
   long long shared_stride;
   long long field_points;

@@ -15,6 +15,8 @@
 // points of one row by adjacent lanes for the contiguous axis).  The spectral
 // product of the convolution (delta-hat x kernel spectrum) is fused into the
 // first pass, the real->complex promotion of delta into the first forward pass.
+#include <algorithm>
+
 #include "sbg_fft_core.cuh"
 
 namespace sbg {
@@ -45,25 +47,28 @@ template <int N, bool CONTIG, int TLV = 0> struct Geo {
 
 template <int N, bool CONTIG, int SIGN, int LOAD, int OUTB, int TLV, bool SLAB>
 __global__ void __launch_bounds__(Geo<N, CONTIG, TLV>::THREADS)
-fft_axis_kernel(FftPass p) {
+fft_axis_kernel(FftPass p, int per_cta) {
   using G = Geo<N, CONTIG, TLV>;
   constexpr int R1 = G::R1, R2 = G::R2, T = G::T, TL = G::TL;
   extern __shared__ float2 sm[];
   const int t = threadIdx.x;
   const int j = CONTIG ? (t % T) : (t / TL);
   const int l = CONTIG ? (t / T) : (t % TL);
-  // Passes with the spectral product run every array of a field in one CTA:
-  // the field's delta-hat values of the CTA's lines are read from HBM once
-  // (into a thread-private shared-memory slot) and reused for each array.
+  // Passes with the spectral product run several transforms of a field in one
+  // CTA (chunk blockIdx.y of per_cta): the field's delta-hat values of the CTA's
+  // lines are read once (into a thread-private shared-memory slot) and reused.
   // Other passes: line group blockIdx.x of batch blockIdx.y.
-  constexpr bool kBins = LOAD == LOAD_MUL || LOAD == LOAD_MUL2;
+  constexpr bool kBins = LOAD == LOAD_MUL || LOAD == LOAD_MUL2 || LOAD == LOAD_MULT;
   const int nbpf = kBins ? (SLAB ? p.nb_per_field : p.batch) : 1;
   unsigned tile = blockIdx.x;
   long long bf0 = 0;  // field of the CTA (kBins)
+  int it0 = 0, it1 = 1;
   if (kBins) {
     const unsigned ntile = (unsigned)(p.outer * (p.inner / TL));
     tile = blockIdx.x % ntile;
     bf0 = blockIdx.x / ntile;
+    it0 = blockIdx.y * per_cta;
+    it1 = min(it0 + per_cta, nbpf);
   }
   float2* sdh = sm + G::SMEM / 8;  // kBins: delta-hat slots, R1 / T x R2 per thread
   long long base;    // element index of point n = 0 of this thread's line
@@ -98,18 +103,24 @@ fft_axis_kernel(FftPass p) {
       for (int n2 = 0; n2 < R2; ++n2)
         sdh[(q * R2 + n2) * G::THREADS + t] = __ldg(p.shared + soff + base + (long long)(j + T * q + R1 * n2) * estride);
   }
+  // the first transform's table entry; the loop loads the next one's ahead, so
+  // that no factor load waits for it
+  constexpr bool kTab = LOAD == LOAD_MUL2 || LOAD == LOAD_MULT;
+  FftXf nxf{0, -1, 0, 0};
+  if (kTab) nxf = p.xf[it0];
+  if (OUTB) nxf = p.xf[SLAB ? blockIdx.y % p.nb_per_field : blockIdx.y];
 #pragma unroll 1
-  for (int it = 0; it < nbpf; ++it) {
+  for (int it = it0; it < it1; ++it) {
+  const FftXf xf = nxf;
+  if (kTab && it + 1 < it1) nxf = p.xf[it + 1];
   const int bat = kBins ? (int)(bf0 * nbpf + it) : (int)blockIdx.y;
   const long long boff = (long long)bat * p.bstride;
-  // batch index = field bf x nb_per_field + array bj of that field (a slab of
-  // fields, SLAB variants); otherwise every batch is array bj of one field
+  // batch index = field bf x nb_per_field + transform bj of that field (a slab
+  // of fields, SLAB variants); otherwise every batch is a transform of one field
   const int bj = SLAB ? bat % p.nb_per_field : bat;
   const long long bf = SLAB ? (long long)bat / p.nb_per_field : 0;
-  const long long moff = (long long)bj * p.bstride;      // factor array of the batch
-  const long long soff = bf * p.shared_stride;            // shared array of its field
   const long long fpts = bf * p.field_points;             // its first point in the blocked store
-  if (it > 0) __syncthreads();  // the previous array's step 2 has read the exchange buffer
+  if (it > it0) __syncthreads();  // the previous array's step 2 has read the exchange buffer
   // opaque per array: the compiler would otherwise keep every point's address
   // and twiddle in registers across the loop (over 160 per thread)
   const float2* twid = p.twiddle;
@@ -121,27 +132,35 @@ fft_axis_kernel(FftPass p) {
   for (int q = 0; q < R1 / T; ++q) {
     const int n1 = j + T * q;
     float2 v[R2];
+    if (kBins) {
+      const float2* ma = p.mul + (long long)(kTab ? xf.a - p.a0 : bj) * p.bstride;
+      const float2* mb = p.mul + (long long)(xf.b - p.a0) * p.bstride;
 #pragma unroll
-    for (int n2 = 0; n2 < R2; ++n2) {
-      const long long e = lbase + (long long)(n1 + R1 * n2) * estride;
-      if (LOAD == LOAD_REAL) {
-        v[n2] = make_float2(__ldg(reinterpret_cast<const float*>(p.in) + boff + e), 0.0f);
-      } else if (LOAD == LOAD_MUL || LOAD == LOAD_MUL2) {
+      for (int n2 = 0; n2 < R2; ++n2) {
+        const long long e = lbase + (long long)(n1 + R1 * n2) * estride;
+        float2 f = __ldg(ma + e);
+        if (LOAD == LOAD_MUL2 && xf.b >= 0) {
+          const float2 g = __ldg(mb + e);
+          f.x -= g.y;
+          f.y += g.x;
+        }
         const float2 dh = sdh[(q * R2 + n2) * G::THREADS + t];
-        if (LOAD == LOAD_MUL) {
-          v[n2] = cmul(dh, __ldg(p.mul + moff + e));
+        if (LOAD == LOAD_MUL2 && N <= 32) {
+          // (the roundings that the compiler's own choice once gave this product;
+          // left to it, they change with the code around them)
+          v[n2] = make_float2(__fmaf_rn(dh.x, f.x, -__fmul_rn(dh.y, f.y)), __fmaf_rn(dh.y, f.x, __fmul_rn(dh.x, f.y)));
         } else {
-          const long long ia = 2 * moff + e;
-          float2 f = __ldg(p.mul + ia);
-          if (2 * bj + 1 < p.npack) {
-            const float2 g = __ldg(p.mul + ia + p.bstride);
-            f.x -= g.y;
-            f.y += g.x;
-          }
           v[n2] = cmul(dh, f);
         }
-      } else {
-        v[n2] = __ldg(reinterpret_cast<const float2*>(p.in) + boff + e);
+      }
+    } else {
+#pragma unroll
+      for (int n2 = 0; n2 < R2; ++n2) {
+        const long long e = lbase + (long long)(n1 + R1 * n2) * estride;
+        if (LOAD == LOAD_REAL)
+          v[n2] = make_float2(__ldg(reinterpret_cast<const float*>(p.in) + boff + e), 0.0f);
+        else
+          v[n2] = __ldg(reinterpret_cast<const float2*>(p.in) + boff + e);
       }
     }
     Dft<R2, SIGN>::run(v);
@@ -162,26 +181,25 @@ fft_axis_kernel(FftPass p) {
 #pragma unroll
     for (int n1 = 0; n1 < R1; ++n1) u[n1] = sm[G::sidx(l, n1, k2)];
     Dft<R1, SIGN>::run(u);
+    if (OUTB) {
 #pragma unroll
-    for (int k1 = 0; k1 < R1; ++k1) {
-      const long long e = lbase + (long long)(k2 + R2 * k1) * estride;
-      if (OUTB == 1) {
-        float* o = reinterpret_cast<float*>(p.out) + blocked_re(fpts + e, p.single0 + bj, p.nsingle);
+      for (int k1 = 0; k1 < R1; ++k1) {
+        const long long e = lbase + (long long)(k2 + R2 * k1) * estride;
+        float* o = reinterpret_cast<float*>(p.out) + blocked_re(fpts + e, xf.s, p.nsingle);
         o[0] = u[k1].x;
-        o[32] = u[k1].y;
-      } else if (OUTB == 2) {
-        const int s = p.single0 + 2 * bj;
-        float* o = reinterpret_cast<float*>(p.out) + blocked_re(fpts + e, s, p.nsingle);
-        o[0] = u[k1].x;
-        o[32] = 0.0f;
-        if (2 * bj + 1 < p.npack) {
-          o = reinterpret_cast<float*>(p.out) + blocked_re(fpts + e, s + 1, p.nsingle);
-          o[0] = u[k1].y;
+        if (OUTB == 1) {
+          o[32] = u[k1].y;
+        } else {
           o[32] = 0.0f;
+          if (xf.b >= 0) {  // single s + 1 follows in the block
+            o[64] = u[k1].y;
+            o[96] = 0.0f;
+          }
         }
-      } else {
-        p.out[boff + e] = u[k1];
       }
+    } else {
+#pragma unroll
+      for (int k1 = 0; k1 < R1; ++k1) p.out[boff + lbase + (long long)(k2 + R2 * k1) * estride] = u[k1];
     }
   }
   }  // arrays of the CTA
@@ -191,7 +209,7 @@ template <int N, bool CONTIG, int SIGN, int LOAD, int OUTB, int TLV, bool SLAB>
 static cudaError_t launch_s(const FftPass& p, cudaStream_t st) {
   using G = Geo<N, CONTIG, TLV>;
   auto kern = fft_axis_kernel<N, CONTIG, SIGN, LOAD, OUTB, TLV, SLAB>;
-  constexpr bool kBins = LOAD == LOAD_MUL || LOAD == LOAD_MUL2;
+  constexpr bool kBins = LOAD == LOAD_MUL || LOAD == LOAD_MUL2 || LOAD == LOAD_MULT;
   constexpr int smem = kBins ? 2 * G::SMEM : G::SMEM;  // + the delta-hat slots
   {
     cudaError_t e = ensure_smem_attr<fft_axis_kernel<N, CONTIG, SIGN, LOAD, OUTB, TLV, SLAB>>(smem);
@@ -202,14 +220,23 @@ static cudaError_t launch_s(const FftPass& p, cudaStream_t st) {
   if (blocks <= 0 || blocks > 0x7fffffffLL || p.batch <= 0 || p.batch > 65535) return cudaErrorInvalidValue;
   if (p.nb_per_field < 0 || (p.nb_per_field && p.batch % p.nb_per_field)) return cudaErrorInvalidValue;
   if (CONTIG ? (p.outer % G::TL) : (p.inner % G::TL)) return cudaErrorInvalidValue;
+  if (OUTB && !p.xf) return cudaErrorInvalidValue;
   dim3 grid((unsigned)blocks, (unsigned)p.batch);
+  int per_cta = 1;
   if constexpr (kBins) {
-    // one CTA per (field, line group), looping over the field's arrays
+    // one CTA per (field, line group) and chunk of the field's transforms: all
+    // of them in one CTA when the line groups alone give every SM 8 CTAs (they
+    // read delta-hat once), else as many chunks as that takes (64^2, 20
+    // transforms: 4 CTAs would hold the whole pass)
     const long long nfld = SLAB ? p.batch / p.nb_per_field : 1;
+    const int ntr = SLAB ? p.nb_per_field : p.batch;
     if (blocks * nfld > 0x7fffffffLL) return cudaErrorInvalidValue;
-    grid = dim3((unsigned)(blocks * nfld), 1u);
+    const long long want = (8LL * device_sms() + blocks * nfld - 1) / (blocks * nfld);
+    const int chunks = (int)std::min<long long>(ntr, std::max<long long>(1, want));
+    per_cta = (ntr + chunks - 1) / chunks;
+    grid = dim3((unsigned)(blocks * nfld), (unsigned)((ntr + per_cta - 1) / per_cta));
   }
-  kern<<<grid, G::THREADS, smem, st>>>(p);
+  kern<<<grid, G::THREADS, smem, st>>>(p, per_cta);
   return cudaGetLastError();
 }
 
@@ -220,7 +247,7 @@ static cudaError_t launch_s(const FftPass& p, cudaStream_t st) {
 // the plain index arithmetic (and its registers).
 template <int N, bool CONTIG, int SIGN, int LOAD, int OUTB, int TLV>
 static cudaError_t launch_v(const FftPass& p, cudaStream_t st) {
-  if constexpr (LOAD == LOAD_MUL || LOAD == LOAD_MUL2 || OUTB != 0)
+  if constexpr (LOAD == LOAD_MUL || LOAD == LOAD_MUL2 || LOAD == LOAD_MULT || OUTB != 0)
     if (p.nb_per_field) return launch_s<N, CONTIG, SIGN, LOAD, OUTB, TLV, true>(p, st);
   return launch_s<N, CONTIG, SIGN, LOAD, OUTB, TLV, false>(p, st);
 }
@@ -231,7 +258,7 @@ static cudaError_t launch_t(const FftPass& p, cudaStream_t st) {
     if (p.tl == 1) return launch_v<N, CONTIG, SIGN, LOAD, OUTB, 1>(p, st);
     // twice the lines at N = 1024 would stage 128 KB per CTA and spill registers;
     // product passes stage their delta-hat values as well (256 KB at N = 512)
-    constexpr bool kBins = LOAD == LOAD_MUL || LOAD == LOAD_MUL2;
+    constexpr bool kBins = LOAD == LOAD_MUL || LOAD == LOAD_MUL2 || LOAD == LOAD_MULT;
     if constexpr (N <= 512 && !(kBins && N >= 512))
       if (p.tl == 2) return launch_v<N, CONTIG, SIGN, LOAD, OUTB, 2>(p, st);
   }
@@ -246,10 +273,7 @@ static cudaError_t dispatch_n(const FftPass& p, cudaStream_t st) {
     if (p.load != LOAD_COMPLEX) return cudaErrorInvalidValue;
     if (p.out_blocked) {
       if (p.sign < 0) return cudaErrorInvalidValue;
-      if (p.out_blocked == 2) {
-        if (p.npack < 1 || p.npack > 2 * p.batch) return cudaErrorInvalidValue;
-        return launch_t<N, true, 1, LOAD_COMPLEX, 2>(p, st);
-      }
+      if (p.out_blocked == 2) return launch_t<N, true, 1, LOAD_COMPLEX, 2>(p, st);
       return launch_t<N, true, 1, LOAD_COMPLEX, 1>(p, st);
     }
     return p.sign < 0 ? launch_t<N, true, -1, LOAD_COMPLEX>(p, st) : launch_t<N, true, 1, LOAD_COMPLEX>(p, st);
@@ -261,10 +285,8 @@ static cudaError_t dispatch_n(const FftPass& p, cudaStream_t st) {
     return cudaErrorInvalidValue;
   }
   if (p.load == LOAD_MUL) return launch_t<N, false, 1, LOAD_MUL>(p, st);
-  if (p.load == LOAD_MUL2) {
-    if (p.npack < 1 || p.npack > 2 * p.batch) return cudaErrorInvalidValue;
-    return launch_t<N, false, 1, LOAD_MUL2>(p, st);
-  }
+  if (p.load == LOAD_MUL2) return p.xf ? launch_t<N, false, 1, LOAD_MUL2>(p, st) : cudaErrorInvalidValue;
+  if (p.load == LOAD_MULT) return p.xf ? launch_t<N, false, 1, LOAD_MULT>(p, st) : cudaErrorInvalidValue;
   if (p.load == LOAD_COMPLEX) return launch_t<N, false, 1, LOAD_COMPLEX>(p, st);
   return cudaErrorInvalidValue;
 }

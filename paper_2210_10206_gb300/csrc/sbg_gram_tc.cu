@@ -165,10 +165,11 @@ __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, i
 
 template <bool TF>
 __global__ void __launch_bounds__(kGThreads, 1)
-gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ a, long long ng, int nb,
+gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, const float* __restrict__ a, long long ng, int gnb, int stack,
+               int ngrp,
                const float* __restrict__ delta,
                double* __restrict__ S, int nsingle, int single0, int* err_flag, unsigned long long wait_ns,
-               int stall, long long s_stride, int gnb, long long g_stride) {
+               int stall, long long s_stride) {
   using C = GramCfg<TF>;
   constexpr int kPts = C::kPts, kFlush = C::kFlush;
   extern __shared__ uint8_t smem_raw[];
@@ -191,13 +192,18 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, const float* __restrict
   volatile int* err = err_flag;
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  // groups blockIdx.z * stack .. of gnb bins each, side by side in one operand
+  const int grp0 = blockIdx.z * stack;
+  const int nb = min(stack, ngrp - grp0) * gnb;
+  single0 += grp0 * gnb;
+  const long long g_stride = 2LL * gnb * gnb;          // doubles of S per group
   const int R = 2 * nb;                                // real rows of W and of U
   const int N = (2 * R + 15) & ~15;                    // MMA N: [U_hi | U_lo] padded
   // field f = blockIdx.y of a slab of fields: its points follow field f - 1's
-  // in the blocked store and delta, its bins in the [field][bin][x] buffer
-  // (rows f nb .. f nb + nb - 1 of the tensor map), its S after field f - 1's
+  // in the blocked store and delta, its arrays in the [field][group][bin][x]
+  // buffer (the rows of the tensor map), its S after field f - 1's
   const int fld = blockIdx.y;
-  S += (long long)fld * s_stride;
+  S += (long long)fld * s_stride + grp0 * g_stride;
   const long long nkb_all = ng / kPts;
   const long long per = (nkb_all + gridDim.x - 1) / gridDim.x;
   const long long kb0 = blockIdx.x * per;
@@ -256,7 +262,7 @@ gram_tc_kernel(const __grid_constant__ CUtensorMap tmap, const float* __restrict
           // rows b = 0 .. nb-1, 128-byte lines x0 / 16 .. x0 / 16 + kPts / 16 - 1
           // (floats 2 x0 .. 2 x0 + 2 kPts - 1), each line's 16-byte chunks
           // swizzled by its line index within the stage
-          tma_load_3d(st, &tmap, 0, (int)(x0 / 16), fld * nb, &raw_full[rs]);
+          tma_load_3d(st, &tmap, 0, (int)(x0 / 16), (fld * ngrp + grp0) * gnb, &raw_full[rs]);
         }
         bulk_g2s(draw + rs * kGDeltaBytes, delta + (long long)fld * ng + x0, (uint32_t)kPts * 4, &raw_full[rs]);
       }
@@ -462,7 +468,7 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 template <bool TF>
 cudaError_t launch_gram_tc_t(const float2* a, long long ng, int nb, const float* delta, double* S, int nsingle,
                              int single0, int* err, int nsm, unsigned long long wait_ns, int stall, int nfld,
-                             long long s_stride, int gnb, long long g_stride, cudaStream_t st) {
+                             long long s_stride, int ngrp, cudaStream_t st) {
   cudaError_t e = ensure_smem_attr<gram_tc_kernel<TF>>(kGSmem);
   if (e != cudaSuccess) return e;
   constexpr int kPts = GramCfg<TF>::kPts;
@@ -477,7 +483,7 @@ cudaError_t launch_gram_tc_t(const float2* a, long long ng, int nb, const float*
     // every row's 2 kPts / 32 lines per K-block, 128-byte swizzled
     PFN_cuTensorMapEncodeTiled_v12000 enc = encode_fn();
     if (!enc || ng / 16 >= (1LL << 31)) return cudaErrorNotSupported;
-    const cuuint64_t dims[3] = {32, (cuuint64_t)(ng / 16), (cuuint64_t)nb * nfld};
+    const cuuint64_t dims[3] = {32, (cuuint64_t)(ng / 16), (cuuint64_t)nb * nfld * ngrp};
     const cuuint64_t strides[2] = {128, (cuuint64_t)ng * 8};
     const cuuint32_t box[3] = {32, (cuuint32_t)(2 * kPts / 32), (cuuint32_t)nb};
     const cuuint32_t estr[3] = {1, 1, 1};
@@ -486,9 +492,9 @@ cudaError_t launch_gram_tc_t(const float2* a, long long ng, int nb, const float*
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) != CUDA_SUCCESS)
       return cudaErrorInvalidValue;
   }
-  gram_tc_kernel<TF><<<dim3(grid, nfld), kGThreads, kGSmem, st>>>(map, (const float*)a, ng, nb, delta, S, nsingle,
-                                                                   single0, err, wait_ns, stall, s_stride, gnb,
-                                                                   g_stride);
+  const int stack = nsingle && ngrp > 1 && 2 * nb <= kGMaxNb ? 2 : 1;
+  gram_tc_kernel<TF><<<dim3(grid, nfld, (ngrp + stack - 1) / stack), kGThreads, kGSmem, st>>>(
+      map, (const float*)a, ng, nb, stack, ngrp, delta, S, nsingle, single0, err, wait_ns, stall, s_stride);
   return cudaGetLastError();
 }
 
@@ -496,15 +502,14 @@ cudaError_t launch_gram_tc_t(const float2* a, long long ng, int nb, const float*
 
 cudaError_t launch_gram_tc(const float2* a, long long ng, int nb, const float* delta, double* S, int nsingle,
                            int single0, int tf32, int* err, int nsm, unsigned long long wait_ns, int stall,
-                           cudaStream_t st, int nfld, long long s_stride, int ngroups, long long g_stride) {
-  if (nb < 1 || nb > kGMaxNb || ng % 64 || !err || nfld < 1 || nfld > 65535) return cudaErrorInvalidValue;
-  if (ngroups < 1 || nb % ngroups || (ngroups > 1 && !nsingle)) return cudaErrorInvalidValue;
-  const int gnb = nb / ngroups;
+                           cudaStream_t st, int nfld, long long s_stride, int ngrp) {
+  if (nb < 1 || nb > kGMaxNb || ng % 64 || !err || nfld < 1 || nfld > 65535 || ngrp < 1 || ngrp > 65535)
+    return cudaErrorInvalidValue;
   if (tf32)
-    return launch_gram_tc_t<true>(a, ng, nb, delta, S, nsingle, single0, err, nsm, wait_ns, stall, nfld, s_stride, gnb,
-                                  g_stride, st);
-  return launch_gram_tc_t<false>(a, ng, nb, delta, S, nsingle, single0, err, nsm, wait_ns, stall, nfld, s_stride, gnb,
-                                 g_stride, st);
+    return launch_gram_tc_t<true>(a, ng, nb, delta, S, nsingle, single0, err, nsm, wait_ns, stall, nfld, s_stride,
+                                  ngrp, st);
+  return launch_gram_tc_t<false>(a, ng, nb, delta, S, nsingle, single0, err, nsm, wait_ns, stall, nfld, s_stride,
+                                 ngrp, st);
 }
 
 }  // namespace sbg

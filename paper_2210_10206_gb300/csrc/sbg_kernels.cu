@@ -126,24 +126,30 @@ __global__ void kgen3d_kernel(int n, int l, int m, double norm, const double* __
   out[(long long)b * ng + cell] = make_float2((float)(s * er), (float)(-s * ei));
 }
 
-// conj(((x + i y)/rho)^m) * Theta_b (Algorithm 2)
-__global__ void kgen2d_kernel(int n, int m, const double* __restrict__ e2, int nb, double scale,
+// conj(((x + i y)/rho)^m) * Theta_b (Algorithm 2) for m = m0 + blockIdx.y, every
+// bin's array written in full (zeros outside the bin)
+__global__ void kgen2d_kernel(int n, int m0, const double* __restrict__ e2, int nb, double scale,
                               float2* __restrict__ out) {
   const long long ng = (long long)n * n;
   const long long cell = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   if (cell >= ng) return;
+  const int m = m0 + blockIdx.y;
+  out += (long long)blockIdx.y * nb * ng;
   const int x = min_image((int)(cell % n), n), y = min_image((int)(cell / n), n);
   const double r2 = (double)x * x + (double)y * y;
   const int b = find_bin(r2, e2, nb);
-  if (b < 0) return;
-  const double r = sqrt(r2);
-  double ur = x / r, ui = y / r, er = 1.0, ei = 0.0;
-  for (int k = 0; k < m; ++k) {
-    const double tr = er * ur - ei * ui;
-    ei = er * ui + ei * ur;
-    er = tr;
+  float2 v = make_float2(0.f, 0.f);
+  if (b >= 0) {
+    const double r = sqrt(r2);
+    double ur = x / r, ui = y / r, er = 1.0, ei = 0.0;
+    for (int k = 0; k < m; ++k) {
+      const double tr = er * ur - ei * ui;
+      ei = er * ui + ei * ur;
+      er = tr;
+    }
+    v = make_float2((float)(er * scale), (float)(-ei * scale));
   }
-  out[(long long)b * ng + cell] = make_float2((float)(er * scale), (float)(-ei * scale));
+  for (int k = 0; k < nb; ++k) out[(long long)k * ng + cell] = k == b ? v : make_float2(0.f, 0.f);
 }
 
 cudaError_t launch_kgen3d(int n, int l, int m, double norm_lm, const double* e2_dev, int nb, double scale,
@@ -153,9 +159,11 @@ cudaError_t launch_kgen3d(int n, int l, int m, double norm_lm, const double* e2_
   return cudaGetLastError();
 }
 
-cudaError_t launch_kgen2d(int n, int m, const double* e2_dev, int nb, double scale, float2* out, cudaStream_t st) {
+cudaError_t launch_kgen2d(int n, int m0, int nm, const double* e2_dev, int nb, double scale, float2* out,
+                          cudaStream_t st) {
   const long long ng = (long long)n * n;
-  kgen2d_kernel<<<(unsigned)((ng + 255) / 256), 256, 0, st>>>(n, m, e2_dev, nb, scale, out);
+  if (nm < 1 || nm > 65535) return cudaErrorInvalidValue;
+  kgen2d_kernel<<<dim3((unsigned)((ng + 255) / 256), (unsigned)nm), 256, 0, st>>>(n, m0, e2_dev, nb, scale, out);
   return cudaGetLastError();
 }
 
@@ -190,12 +198,14 @@ __device__ __forceinline__ void gram_cp(void* dst, const void* src, bool ok, int
 __global__ void __launch_bounds__(512, 2) gram3_kernel(const float2* __restrict__ a, long long ng, int nb,
                                                     const float* __restrict__ delta, double* __restrict__ S,
                                                     int nsingle, int single0, long long s_stride) {
-  // field f = blockIdx.y of a slab: its bins follow field f - 1's (group
-  // buffer) or its points do (blocked store); its delta and S likewise
+  // field f = blockIdx.y of a slab: its arrays follow field f - 1's (group
+  // buffer) or its points do (blocked store); its delta and S likewise.  Group
+  // blockIdx.z: the next nb arrays or singles, and the next S block
   const long long fx = (long long)blockIdx.y * ng;
-  if (!nsingle) a += (long long)blockIdx.y * nb * ng;
+  if (!nsingle) a += ((long long)blockIdx.y * gridDim.z + blockIdx.z) * nb * ng;
+  single0 += blockIdx.z * nb;
   delta += fx;
-  S += (long long)blockIdx.y * s_stride;
+  S += (long long)blockIdx.y * s_stride + (long long)blockIdx.z * nb * nb * 2;
   const int nbb = (nb + 3) / 4, nrow = 4 * nbb;
   // stage: nrow rows of kGramChunk (re, im), then kGramChunk deltas; rows nb ..
   // of the last block stay zero
@@ -334,8 +344,8 @@ __global__ void __launch_bounds__(512, 2) gram3_kernel(const float2* __restrict_
 }
 
 cudaError_t launch_gram3(const float2* a, long long ng, int nb, const float* delta, double* S, int nsingle,
-                         int single0, cudaStream_t st, int nfld, long long s_stride) {
-  if (nb < 1 || nb > kGramMaxNb || nfld < 1 || nfld > 65535) return cudaErrorInvalidValue;
+                         int single0, cudaStream_t st, int nfld, long long s_stride, int ngrp) {
+  if (nb < 1 || nb > kGramMaxNb || nfld < 1 || nfld > 65535 || ngrp < 1 || ngrp > 65535) return cudaErrorInvalidValue;
   // 16-byte copies of the group buffer and of delta
   if (!nsingle && (((uintptr_t)a & 15) || (ng & 1))) return cudaErrorInvalidValue;
   if (((uintptr_t)delta & 15) || (ng & 3)) return cudaErrorInvalidValue;
@@ -352,7 +362,7 @@ cudaError_t launch_gram3(const float2* a, long long ng, int nb, const float* del
   if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gram3_kernel, threads, smem)) != cudaSuccess) return e;
   const long long cap = std::max<long long>(1, ((long long)device_sms() * std::max(per_sm, 1) + nfld - 1) / nfld);
   if (blocks > cap) blocks = cap;
-  gram3_kernel<<<dim3((unsigned)blocks, nfld), threads, smem, st>>>(a, ng, nb, delta, S, nsingle, single0, s_stride);
+  gram3_kernel<<<dim3((unsigned)blocks, nfld, ngrp), threads, smem, st>>>(a, ng, nb, delta, S, nsingle, single0, s_stride);
   return cudaGetLastError();
 }
 

@@ -16,8 +16,9 @@ cudaError_t launch_convert(const void* in, int is_f64, long long n, const double
 // 3D: out[b][cell] = conj(Y_lm(r_hat)) Theta_b(|r|) * scale for b < nb (buffer pre-zeroed).
 cudaError_t launch_kgen3d(int n, int l, int m, double norm_lm, const double* e2_dev, int nb, double scale,
                           float2* out, cudaStream_t st);
-// 2D: out[b][cell] = conj(((x+iy)/rho)^m) Theta_b(rho) * scale.
-cudaError_t launch_kgen2d(int n, int m, const double* e2_dev, int nb, double scale, float2* out,
+// 2D: out[k][b][cell] = conj(((x+iy)/rho)^m) Theta_b(rho) * scale, m = m0 + k, for
+// k < nm; every element is written.
+cudaError_t launch_kgen2d(int n, int m0, int nm, const double* e2_dev, int nb, double scale, float2* out,
                           cudaStream_t st);
 
 // ---- 3PCF Gram (Eq. alm_to_zeta_clean / proj_3pcf_coeff, Algorithms 5 and 7) ----
@@ -25,10 +26,11 @@ cudaError_t launch_kgen2d(int n, int m, const double* e2_dev, int nb, double sca
 // nsingle > 0: `a` is the blocked coefficient store and bin b is single single0 + b;
 // nsingle = 0: `a` is [nb][ng].
 // A slab of nfld fields of ng points: field f's bins follow field f - 1's in
-// the [field][bin][x] buffer (nsingle = 0) or its points follow in the blocked
-// store; delta + f ng; S + f s_stride (doubles).
+// the [field][group][bin][x] buffer (nsingle = 0) or its points follow in the
+// blocked store; delta + f ng; S + f s_stride (doubles).  ngrp groups of nb
+// bins, adjacent in the store or buffer, add into S blocks of nb nb complex each.
 cudaError_t launch_gram3(const float2* a, long long ng, int nb, const float* delta, double* S, int nsingle,
-                         int single0, cudaStream_t st, int nfld = 1, long long s_stride = 0);
+                         int single0, cudaStream_t st, int nfld = 1, long long s_stride = 0, int ngrp = 1);
 
 // ---- 4PCF pair x single contraction tables (Algorithms 6 and 8) ----
 struct Tile4 {
@@ -121,14 +123,13 @@ cudaError_t launch_tc4(const float2* astore, void* bimg, const BGroup* bgroups, 
 // multiple of 64.  *err is set (never cleared) if a bounded wait (wait_ns of
 // the GPU's global timer) expired; stall != 0 withholds its MMA issuer (a
 // host-side test of the timeout path).
-// Slabs of nfld fields as for launch_gram3.  With ngroups > 1 (blocked store
-// only) the nb singles from single0 are ngroups adjacent groups of nb / ngroups
-// bins: only pairs within one group are kept, group k's S at S + k * g_stride.
+// Slabs of nfld fields and ngrp groups as for launch_gram3.  Two adjacent groups
+// of at most 10 bins in the blocked store share a CTA's pass (their 2 nb singles
+// are one operand; only the pairs within a group are kept).
 constexpr int kGramTcMaxNb = 20;
 cudaError_t launch_gram_tc(const float2* a, long long ng, int nb, const float* delta, double* S, int nsingle,
                            int single0, int tf32, int* err, int nsm, unsigned long long wait_ns, int stall,
-                           cudaStream_t st, int nfld = 1, long long s_stride = 0, int ngroups = 1,
-                           long long g_stride = 0);
+                           cudaStream_t st, int nfld = 1, long long s_stride = 0, int ngrp = 1);
 
 // ---- kernel generation fused with the FFT (sbg_fft_fused.cu) ----
 // One (l, m) group of nb bins of a 3D grid of side n whose kernel spectra are

@@ -8,6 +8,7 @@
 // one file-scope __device__ array (kScratchBytes per device that loads this
 // library, held until the process exits).  The caller passes the field and the
 // output as device pointers.
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <cstring>
@@ -29,7 +30,9 @@ constexpr size_t kOffE2 = kOffAcc + up(8 * 8);                               // 
 constexpr size_t kOffTw = kOffE2 + up((kMaxBins + 1) * 8);                   // N float2
 constexpr size_t kOffDelta = kOffTw + up((size_t)kMaxN * 8);                 // N^2 floats
 constexpr size_t kOffDhat = kOffDelta + up((size_t)kMaxN * kMaxN * 4);       // N^2 float2
-constexpr size_t kOffG = kOffDhat + up((size_t)kMaxN * kMaxN * 8);           // nbins N^2 float2
+// kernel spectra and coefficients: kMaxBins arrays of kMaxN^2 each, or as many
+// groups (orders m) of smaller ones as fit
+constexpr size_t kOffG = kOffDhat + up((size_t)kMaxN * kMaxN * 8);           // float2
 constexpr size_t kOffGroup = kOffG + up((size_t)kMaxBins * kMaxN * kMaxN * 8);
 constexpr size_t kOffS = kOffGroup + up((size_t)kMaxBins * kMaxN * kMaxN * 8);
 constexpr size_t kScratchBytes = kOffS + up((size_t)(kMaxM + 1) * kMaxBins * kMaxBins * 16);
@@ -70,9 +73,12 @@ struct HostTables {
   int nbins, n;
 };
 
-__global__ void tables_kernel(const HostTables t, double* e2d, float2* tw) {
+// also clears the accumulators (the array keeps the previous call's contents)
+__global__ void tables_kernel(const HostTables t, double* e2d, float2* tw, double* acc, double* S, int nS) {
   for (int i = threadIdx.x; i < t.n; i += blockDim.x) tw[i] = t.tw[i];
   if ((int)threadIdx.x <= t.nbins) e2d[threadIdx.x] = t.e2[threadIdx.x];
+  if (threadIdx.x < 8) acc[threadIdx.x] = 0.0;
+  for (int i = threadIdx.x; i < nS; i += blockDim.x) S[i] = 0.0;
 }
 
 #define NA_CU(call)                         \
@@ -129,11 +135,8 @@ extern "C" sbg_status sbg_projected3_noalloc(const void* field, sbg_dtype dtype,
     const double a = 2.0 * 3.14159265358979323846 * j / N;
     ht.tw[j] = make_float2((float)std::cos(a), (float)std::sin(a));
   }
-  tables_kernel<<<1, 256, 0, stream>>>(ht, e2d, tw);
+  tables_kernel<<<1, 256, 0, stream>>>(ht, e2d, tw, acc, S, (mmax + 1) * nbins * nbins * 2);
   NA_CU(cudaGetLastError());
-  // the array keeps the previous call's contents: clear the accumulators
-  NA_CU(cudaMemsetAsync(acc, 0, 8 * sizeof(double), stream));
-  NA_CU(cudaMemsetAsync(S, 0, (size_t)(mmax + 1) * nbins * nbins * 16, stream));
 
   NA_CU(launch_sum(field, dtype == SBG_F64, ng, acc, stream));
   NA_CU(launch_convert(field, dtype == SBG_F64, ng, acc, (flags & SBG_SUBTRACT_MEAN) ? 1 : 0, delta, stream));
@@ -145,24 +148,28 @@ extern "C" sbg_status sbg_projected3_noalloc(const void* field, sbg_dtype dtype,
   NA_CU(fft_axis_pass(N, p, stream));
   p.in = dhat; p.load = LOAD_COMPLEX; p.outer = N; p.inner = 1;
   NA_CU(fft_axis_pass(N, p, stream));
-  for (int m = 0; m <= mmax; ++m) {
+  // the orders m in steps of as many groups as the scratch arrays hold: every
+  // stage is one launch for all of a step's groups (128^2, 7 bins, mmax 5: 19
+  // launches instead of 47)
+  const int step = std::min(mmax + 1, (int)((long long)kMaxBins * kMaxN * kMaxN / (nbins * ng)));
+  for (int m = 0; m <= mmax; m += step) {
+    const int k = std::min(step, mmax + 1 - m), arrays = k * nbins;
     // kernel spectra G^b_m = FFT_+(conj(e^{i m phi}) Theta_b) / N^2
-    NA_CU(cudaMemsetAsync(G, 0, (size_t)nbins * ng * sizeof(float2), stream));
-    NA_CU(launch_kgen2d(N, m, e2d, nbins, 1.0 / (double)ng, G, stream));
+    NA_CU(launch_kgen2d(N, m, k, e2d, nbins, 1.0 / (double)ng, G, stream));
     FftPass q{};
-    q.twiddle = tw; q.batch = nbins; q.bstride = ng; q.sign = +1;
+    q.twiddle = tw; q.batch = arrays; q.bstride = ng; q.sign = +1;
     q.in = G; q.out = G; q.load = LOAD_COMPLEX; q.outer = 1; q.inner = N;
     NA_CU(fft_axis_pass(N, q, stream));
     q.outer = N; q.inner = 1;
     NA_CU(fft_axis_pass(N, q, stream));
     // c^b_m = IFFT(delta-hat G^b_m), product fused into the first pass
     FftPass c{};
-    c.twiddle = tw; c.batch = nbins; c.bstride = ng; c.sign = +1;
+    c.twiddle = tw; c.batch = arrays; c.bstride = ng; c.sign = +1;
     c.out = grp; c.mul = G; c.shared = dhat; c.load = LOAD_MUL; c.outer = 1; c.inner = N;
     NA_CU(fft_axis_pass(N, c, stream));
     c.in = grp; c.mul = nullptr; c.shared = nullptr; c.load = LOAD_COMPLEX; c.outer = N; c.inner = 1;
     NA_CU(fft_axis_pass(N, c, stream));
-    NA_CU(launch_gram3(grp, ng, nbins, delta, S + (size_t)m * nbins * nbins * 2, 0, 0, stream));
+    NA_CU(launch_gram3(grp, ng, nbins, delta, S + (size_t)m * nbins * nbins * 2, 0, 0, stream, 1, 0, k));
   }
   NA_CU(launch_finish3(S, 0, mmax, nbins, zeta3, stream));
   return SBG_OK;

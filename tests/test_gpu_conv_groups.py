@@ -1,0 +1,53 @@
+"""Convolutions and Grams of several (l, m) or m groups per launch against one
+group per launch (a context with a memory budget takes one): the transforms and
+the FP32 / tensor-core sums are the same operations in the same order, so the
+outputs differ by the order of FP64 reductions only: <= 1e-12 of max |zeta|."""
+import numpy as np
+import pytest
+
+from paper_2210_10206_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+TOL = 1e-12
+
+
+@pytest.fixture(scope="module")
+def pair():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2210_10206_gb300 import build, sbg
+    build.build()
+    c = sbg.Context(0), sbg.Context(0, budget=2 << 30)
+    yield c
+    for x in c:
+        x.close()
+
+
+def _same(a, b):
+    for x, y in zip(a, b):
+        if x is not None:
+            assert np.abs(x - y).max() <= TOL * np.abs(y).max()
+
+
+@pytest.mark.parametrize("prec", [0, 1, 3])
+@pytest.mark.parametrize("n,nb,mmax,npcf", [(8, 1, 0, (3, 4)), (16, 3, 4, (3, 4)), (64, 10, 5, (3,)), (128, 5, 10, (3, 4)),
+                                            (1024, 2, 3, (3, 4))])
+def test_projected(pair, n, nb, mmax, npcf, prec):
+    f = synth.lognormal_field(800 + n, (n, n), 1.0, -2.0)
+    edges = np.linspace(0.5, min(0.46 * n, 60.0), nb + 1)
+    _same(*[c.projected(f, edges, mmax, npcf=npcf, prec=prec) for c in pair])
+
+
+@pytest.mark.parametrize("prec", [0, 1])
+@pytest.mark.parametrize("n,nb,lmax3,lmax4", [(8, 1, 0, 0), (16, 3, 2, 3), (32, 5, 3, 1), (64, 2, None, 2)])
+def test_full(pair, n, nb, lmax3, lmax4, prec):
+    f = synth.lognormal_field(820 + n, (n, n, n), 1.0, -2.0)
+    edges = np.linspace(0.5, min(0.46 * n, 16.0), nb + 1)
+    _same(*[c.full(f, edges, lmax3=lmax3, lmax4=lmax4, prec=prec) for c in pair])
+
+
+@pytest.mark.parametrize("npcf", [(3,), (3, 4)])
+def test_slab(pair, npcf):
+    cube = np.stack([synth.lognormal_field(840 + i, (32, 32), 1.0, -2.0) for i in range(5)])
+    _same(*[c.projected_slices(cube, np.linspace(0.5, 14.0, 8), 3, npcf=npcf) for c in pair])
