@@ -14,7 +14,9 @@
 #include <cstring>
 #include <map>
 #include <queue>
+#include <set>
 #include <string>
+#include <system_error>
 #include <thread>
 #include <tuple>
 #include <unordered_map>
@@ -190,7 +192,14 @@ struct sbg_context {
   };
   bool defer = false;
   int cur = 0;
-  std::string xf_key;  // what the transform table in buffer "xf" was made for
+  // host tables that the device already holds (see Tables): what the transform
+  // table in buffer "xf" was made for, the sides whose twiddles are uploaded, the
+  // squared edges, and the support lines of (side, outermost squared edge)
+  std::string xf_key;
+  std::set<int> tw_sides;
+  std::vector<double> e2_up;
+  std::pair<int, double> lines_key{0, 0.0};
+  int nlines = 0, rsup = 0;
   // autotuner: launch choices measured on their first use, by key
   std::map<std::string, int> tune;
   cudaEvent_t tev[2] = {};
@@ -1292,6 +1301,78 @@ sbg_status finish_timings(sbg_context* ctx) {
   return SBG_OK;
 }
 
+// Uploads of small host tables are skipped while the device holds the same ones
+// (each costs several microseconds of host time before the first kernel).  A call
+// that fails forgets them: its queued uploads may not have run.
+struct TableGuard {
+  sbg_context* ctx;
+  bool ok = false;
+  ~TableGuard() {
+    if (ok) return;
+    ctx->xf_key.clear();
+    ctx->tw_sides.clear();
+    ctx->e2_up.clear();
+    ctx->lines_key = {0, 0.0};
+  }
+};
+
+// Twiddles of side n, squared edges and (normalised calls only) bin volumes.
+sbg_status geometry_tables(sbg_context* ctx, int n, const std::vector<double>& e2, const std::vector<double>& vb, float2** tw,
+                           double** d_e2, double** d_vb) {
+  const std::string name = "tw" + std::to_string(n);
+  ST(buf(ctx, name.c_str(), n * 8, (void**)tw));
+  ST(buf(ctx, "e2", (kMaxBins + 1) * 8, (void**)d_e2));
+  ST(buf(ctx, "vb", kMaxBins * 8, (void**)d_vb));
+  if (!ctx->tw_sides.count(n)) {
+    const std::vector<float2> t = twiddles(n);
+    CU(cudaMemcpyAsync(*tw, t.data(), n * 8, cudaMemcpyHostToDevice, ctx->stream));
+    ctx->tw_sides.insert(n);
+  }
+  if (ctx->e2_up != e2) {
+    ctx->e2_up.clear();
+    CU(cudaMemcpyAsync(*d_e2, e2.data(), e2.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
+    ctx->e2_up = e2;
+  }
+  if (!vb.empty()) CU(cudaMemcpyAsync(*d_vb, vb.data(), vb.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
+  return SBG_OK;
+}
+
+// Copies of results from pinned staging to the caller's arrays, by up to 8 host
+// threads of at least 512 KB each: a fresh result array's page faults cost more
+// than the copy (15.5 MB: 1.5 ms on one thread).
+struct HostCopy {
+  void* dst;
+  const void* src;
+  size_t bytes;
+};
+void copy_out(const std::vector<HostCopy>& c) {
+  size_t total = 0;
+  for (const HostCopy& x : c) total += x.bytes;
+  auto part = [&](size_t b0, size_t b1) {  // bytes [b0, b1) of the copies in a row
+    size_t at = 0;
+    for (const HostCopy& x : c) {
+      const size_t lo = std::max(b0, at), hi = std::min(b1, at + x.bytes);
+      if (lo < hi) std::memcpy((char*)x.dst + (lo - at), (const char*)x.src + (lo - at), hi - lo);
+      at += x.bytes;
+    }
+  };
+  const size_t hw = std::max(1u, std::thread::hardware_concurrency());
+  const size_t nt = std::max<size_t>(1, std::min<size_t>({8, hw, total / (512u << 10)}));
+  const size_t per = (total / nt + 4095) / 4096 * 4096;
+  std::vector<std::thread> th;
+  for (size_t t = 1; t < nt; ++t) {
+    // without a thread to be had, this one does the rest
+    try {
+      th.emplace_back(part, t * per, t + 1 == nt ? total : (t + 1) * per);
+    } catch (const std::system_error&) {
+      part(t * per, total);
+      break;
+    }
+  }
+  part(0, nt == 1 ? total : per);
+  for (auto& x : th) x.join();
+}
+
 // ---------------------------------------------------------------- core ----
 // Shared by sbg_full (dim 3) and sbg_projected / batch (dim 2).
 // odd (dim 3, 4PCF only): the odd-parity Lambda, zeta4 receives Im of each coefficient
@@ -1306,12 +1387,12 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
   const int ngroups = npair(L);
   const int ngroups4 = do4 ? npair(lmax4) : 0;
   const std::vector<double> e2 = snap_e2(edges, nb);
-  const std::vector<double> vb = cell_counts(n, dim, e2, nb);
+  TableGuard tables{ctx};
+  const std::vector<double> vb = flags & SBG_NORMALIZED ? cell_counts(n, dim, e2, nb) : std::vector<double>();
   if (flags & SBG_NORMALIZED)
     for (int b = 0; b < nb; ++b)
       if (vb[b] == 0.0) return fail(ctx, SBG_ERR_EMPTY_BIN, "bin " + std::to_string(b) + " holds no cell");
 
-  for (int i = 0; i <= kStages; ++i) rec(ctx, i);  // reset
   ctx->kev_used = false;
   ctx->nlaunch = 0;
   rec(ctx, 0);
@@ -1330,15 +1411,7 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
   ST(buf(ctx, "delta", ng * 4, (void**)&d_delta));
   ST(buf(ctx, "dhat", ng * 8, (void**)&d_dhat));
   ST(buf(ctx, "acc", 64, (void**)&d_acc));
-  ST(buf(ctx, "tw", n * 8, (void**)&d_tw));
-  ST(buf(ctx, "e2", (kMaxBins + 1) * 8, (void**)&d_e2));
-  ST(buf(ctx, "vb", kMaxBins * 8, (void**)&d_vb));
-  {
-    const std::vector<float2> tw = twiddles(n);
-    CU(cudaMemcpyAsync(d_tw, tw.data(), n * 8, cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(d_e2, e2.data(), (nb + 1) * 8, cudaMemcpyHostToDevice, ctx->stream));
-    CU(cudaMemcpyAsync(d_vb, vb.data(), nb * 8, cudaMemcpyHostToDevice, ctx->stream));
-  }
+  ST(geometry_tables(ctx, n, e2, vb, &d_tw, &d_e2, &d_vb));
   CU(cudaMemsetAsync(d_acc, 0, 64, ctx->stream));
   KL(launch_sum(d_in, dtype == SBG_F64, ng, d_acc, ctx->stream));
   KL(launch_convert(d_in, dtype == SBG_F64, ng, d_acc, (flags & SBG_SUBTRACT_MEAN) ? 1 : 0, d_delta, ctx->stream));
@@ -1430,16 +1503,25 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
   int* d_lines = nullptr;
   int nlines = 0, Rsup = 0;
   if (fused) {
-    std::vector<int> lines;
-    for (int zi = 0; zi < n; ++zi)
-      for (int yi = 0; yi < n; ++yi) {
-        const double z = zi < n - zi ? zi : zi - n, y = yi < n - yi ? yi : yi - n;
-        if (y * y + z * z <= e2[nb]) lines.push_back(zi * n + yi);
-      }
-    while ((double)(Rsup + 1) * (Rsup + 1) <= e2[nb]) ++Rsup;
-    nlines = (int)lines.size();
-    ST(buf(ctx, "klines", std::max<size_t>(lines.size(), 1) * 4, (void**)&d_lines));
-    if (nlines) CU(cudaMemcpyAsync(d_lines, lines.data(), lines.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
+    if (ctx->lines_key != std::make_pair(n, e2[nb])) {
+      ctx->lines_key = {0, 0.0};
+      std::vector<int> lines;
+      for (int zi = 0; zi < n; ++zi)
+        for (int yi = 0; yi < n; ++yi) {
+          const double z = zi < n - zi ? zi : zi - n, y = yi < n - yi ? yi : yi - n;
+          if (y * y + z * z <= e2[nb]) lines.push_back(zi * n + yi);
+        }
+      ctx->rsup = 0;
+      while ((double)(ctx->rsup + 1) * (ctx->rsup + 1) <= e2[nb]) ++ctx->rsup;
+      ctx->nlines = (int)lines.size();
+      ST(buf(ctx, "klines", std::max<size_t>(lines.size(), 1) * 4, (void**)&d_lines));
+      if (ctx->nlines)
+        CU(cudaMemcpyAsync(d_lines, lines.data(), lines.size() * 4, cudaMemcpyHostToDevice, ctx->stream));
+      ctx->lines_key = {n, e2[nb]};
+    }
+    nlines = ctx->nlines;
+    Rsup = ctx->rsup;
+    ST(buf(ctx, "klines", (size_t)std::max(nlines, 1) * 4, (void**)&d_lines));
   }
   // delta-weighted Grams of the groups [g0, g1) in one launch: from the blocked
   // store, or from the group buffer
@@ -1648,11 +1730,15 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
     pd.b4 = z4bytes;
     pd.launches = ctx->nlaunch;
     pd.kev_used = ctx->kev_used;
+    tables.ok = true;
     return SBG_OK;
   }
   ST(finish_timings(ctx));
-  if (do3) std::memcpy(zeta3, hst + z3off, z3bytes);
-  if (do4) std::memcpy(zeta4, hst + z4off, z4bytes);
+  std::vector<HostCopy> copies;
+  if (do3) copies.push_back({zeta3, hst + z3off, z3bytes});
+  if (do4) copies.push_back({zeta4, hst + z4off, z4bytes});
+  copy_out(copies);
+  tables.ok = true;
   return SBG_OK;
 }
 
@@ -1681,7 +1767,8 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
   const int ngroups = mmax + 1;
   const int ngroups4 = do4 ? mmax + 1 : 0;
   const std::vector<double> e2 = snap_e2(edges, nb);
-  const std::vector<double> vb = cell_counts(n, 2, e2, nb);
+  TableGuard tables{ctx};
+  const std::vector<double> vb = flags & SBG_NORMALIZED ? cell_counts(n, 2, e2, nb) : std::vector<double>();
   if (flags & SBG_NORMALIZED)
     for (int b = 0; b < nb; ++b)
       if (vb[b] == 0.0) return fail(ctx, SBG_ERR_EMPTY_BIN, "bin " + std::to_string(b) + " holds no cell");
@@ -1713,15 +1800,7 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
   ST(buf(ctx, "delta", (size_t)nfld * ng * 4, (void**)&d_delta));
   ST(buf(ctx, "dhat", (size_t)nfld * ng * 8, (void**)&d_dhat));
   ST(buf(ctx, "acc", (size_t)std::max(64, 16 * nfld), (void**)&d_acc));
-  ST(buf(ctx, "tw", n * 8, (void**)&d_tw));
-  ST(buf(ctx, "e2", (kMaxBins + 1) * 8, (void**)&d_e2));
-  ST(buf(ctx, "vb", kMaxBins * 8, (void**)&d_vb));
-  {
-    const std::vector<float2> tw = twiddles(n);
-    CU(cudaMemcpyAsync(d_tw, tw.data(), n * 8, cudaMemcpyHostToDevice, st));
-    CU(cudaMemcpyAsync(d_e2, e2.data(), (nb + 1) * 8, cudaMemcpyHostToDevice, st));
-    CU(cudaMemcpyAsync(d_vb, vb.data(), nb * 8, cudaMemcpyHostToDevice, st));
-  }
+  ST(geometry_tables(ctx, n, e2, vb, &d_tw, &d_e2, &d_vb));
   CU(cudaMemsetAsync(d_acc, 0, (size_t)16 * nfld, st));
   KL(launch_sum(d_in, dtype == SBG_F64, ng, d_acc, st, nfld));
   KL(launch_convert(d_in, dtype == SBG_F64, ng, d_acc, (flags & SBG_SUBTRACT_MEAN) ? 1 : 0, d_delta, st, nfld));
@@ -1928,30 +2007,18 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
   out->z4b = z4b;
   out->off4 = off4;
   out->host = hslot;
+  tables.ok = true;
   return SBG_OK;
 }
 
-// Copies a slab's results from the pinned slot to the fields' arrays, with
-// several host threads when there is much to copy (the dense 4PCF outputs of a
-// slab of slices reach hundreds of MB).
+// Copies a slab's results from the pinned slot to the fields' arrays.
 void slab_copy_out(const SlabOut& o) {
-  auto part = [&o](int f0, int f1) {
-    for (int i = f0; i < f1; ++i) {
-      if (o.z3b && o.fields[i].zeta3) std::memcpy(o.fields[i].zeta3, o.host + (size_t)i * o.z3b, o.z3b);
-      if (o.z4b && o.fields[i].zeta4) std::memcpy(o.fields[i].zeta4, o.host + o.off4 + (size_t)i * o.z4b, o.z4b);
-    }
-  };
-  const size_t total = (size_t)o.nfld * (o.z3b + o.z4b);
-  const unsigned hw = std::max(1u, std::thread::hardware_concurrency());
-  const int nt = (int)std::min<size_t>({(size_t)8, (size_t)hw, (size_t)o.nfld, total / (16u << 20) + 1});
-  if (nt <= 1) {
-    part(0, o.nfld);
-    return;
+  std::vector<HostCopy> c;
+  for (int i = 0; i < o.nfld; ++i) {
+    if (o.z3b && o.fields[i].zeta3) c.push_back({o.fields[i].zeta3, o.host + (size_t)i * o.z3b, o.z3b});
+    if (o.z4b && o.fields[i].zeta4) c.push_back({o.fields[i].zeta4, o.host + o.off4 + (size_t)i * o.z4b, o.z4b});
   }
-  std::vector<std::thread> th;
-  for (int t = 1; t < nt; ++t) th.emplace_back(part, o.nfld * t / nt, o.nfld * (t + 1) / nt);
-  part(0, o.nfld / nt);
-  for (auto& x : th) x.join();
+  copy_out(c);
 }
 
 }  // namespace
