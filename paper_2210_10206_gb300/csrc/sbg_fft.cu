@@ -45,7 +45,12 @@ template <int N, bool CONTIG, int TLV = 0> struct Geo {
   }
 };
 
-template <int N, bool CONTIG, int SIGN, int LOAD, int OUTB, int TLV, bool SLAB>
+// AX: the stride along a strided line, known to the compiler where that matters (1:
+// N, lines along y; 2: N^2, lines along z; 0: p.inner).  With a run-time stride the
+// N >= 512 passes kept 32 addresses in 174 registers, one CTA per SM; with a
+// constant one they take 90 and run three: 512^3 y pass 4.8 -> 7.1 TB/s, z pass 4.5
+// -> 6.5, 1024^2 product pass 2.8 -> 4.2 (copy 6.7; N <= 256 has run at 6.4 to 7.2).
+template <int N, bool CONTIG, int SIGN, int LOAD, int OUTB, int TLV, bool SLAB, int AX>
 __global__ void __launch_bounds__(Geo<N, CONTIG, TLV>::THREADS)
 fft_axis_kernel(FftPass p, int per_cta) {
   using G = Geo<N, CONTIG, TLV>;
@@ -72,10 +77,9 @@ fft_axis_kernel(FftPass p, int per_cta) {
   }
   float2* sdh = sm + G::SMEM / 8;  // kBins: delta-hat slots, R1 / T x R2 per thread
   long long base;    // element index of point n = 0 of this thread's line
-  long long estride; // element stride along the line
+  const long long estride = CONTIG ? 1 : AX == 1 ? N : AX == 2 ? (long long)N * N : p.inner;  // along the line
   if (CONTIG) {
     base = ((long long)tile * TL + l) * N;
-    estride = 1;
   } else {
     const long long tiles = p.inner / TL;
     const long long o = tile / tiles;
@@ -91,10 +95,13 @@ fft_axis_kernel(FftPass p, int per_cta) {
       if (zero) return;
     }
     base = o * (long long)N * p.inner + i0 + l;
-    estride = p.inner;
   }
 
-  if (kBins) {
+  // at N = 1024 (2D) delta-hat comes from L2 for every transform: a slot would take
+  // the CTA's shared memory to 128 KB, one CTA per SM
+  constexpr bool kSlot = kBins && N < 1024;
+  const float2* dsh = p.shared + (SLAB ? bf0 : 0LL) * p.shared_stride;
+  if (kSlot) {
     // this thread's delta-hat values (the points it loads in step 1), once
     const long long soff = (SLAB ? bf0 : 0LL) * p.shared_stride;
 #pragma unroll
@@ -144,7 +151,7 @@ fft_axis_kernel(FftPass p, int per_cta) {
           f.x -= g.y;
           f.y += g.x;
         }
-        const float2 dh = sdh[(q * R2 + n2) * G::THREADS + t];
+        const float2 dh = kSlot ? sdh[(q * R2 + n2) * G::THREADS + t] : __ldg(dsh + e);
         if (LOAD == LOAD_MUL2 && N <= 32) {
           // (the roundings that the compiler's own choice once gave this product;
           // left to it, they change with the code around them)
@@ -205,14 +212,14 @@ fft_axis_kernel(FftPass p, int per_cta) {
   }  // arrays of the CTA
 }
 
-template <int N, bool CONTIG, int SIGN, int LOAD, int OUTB, int TLV, bool SLAB>
-static cudaError_t launch_s(const FftPass& p, cudaStream_t st) {
+template <int N, bool CONTIG, int SIGN, int LOAD, int OUTB, int TLV, bool SLAB, int AX>
+static cudaError_t launch_u(const FftPass& p, cudaStream_t st) {
   using G = Geo<N, CONTIG, TLV>;
-  auto kern = fft_axis_kernel<N, CONTIG, SIGN, LOAD, OUTB, TLV, SLAB>;
+  auto kern = fft_axis_kernel<N, CONTIG, SIGN, LOAD, OUTB, TLV, SLAB, AX>;
   constexpr bool kBins = LOAD == LOAD_MUL || LOAD == LOAD_MUL2 || LOAD == LOAD_MULT;
-  constexpr int smem = kBins ? 2 * G::SMEM : G::SMEM;  // + the delta-hat slots
+  constexpr int smem = kBins && N < 1024 ? 2 * G::SMEM : G::SMEM;  // + the delta-hat slots
   {
-    cudaError_t e = ensure_smem_attr<fft_axis_kernel<N, CONTIG, SIGN, LOAD, OUTB, TLV, SLAB>>(smem);
+    cudaError_t e = ensure_smem_attr<fft_axis_kernel<N, CONTIG, SIGN, LOAD, OUTB, TLV, SLAB, AX>>(smem);
     if (e != cudaSuccess) return e;
   }
   // contiguous: outer rows grouped by TL; strided: outer * inner lines grouped by TL
@@ -238,6 +245,16 @@ static cudaError_t launch_s(const FftPass& p, cudaStream_t st) {
   }
   kern<<<grid, G::THREADS, smem, st>>>(p, per_cta);
   return cudaGetLastError();
+}
+
+template <int N, bool CONTIG, int SIGN, int LOAD, int OUTB, int TLV, bool SLAB>
+static cudaError_t launch_s(const FftPass& p, cudaStream_t st) {
+  if constexpr (!CONTIG && N >= 512)
+    if (p.inner == N) return launch_u<N, CONTIG, SIGN, LOAD, OUTB, TLV, SLAB, 1>(p, st);
+  if constexpr (!CONTIG && N == 512 && !SLAB)
+    if (p.inner == N * N) return launch_u<N, CONTIG, SIGN, LOAD, OUTB, TLV, SLAB, 2>(p, st);
+  if constexpr (CONTIG || N < 512) return launch_u<N, CONTIG, SIGN, LOAD, OUTB, TLV, SLAB, 0>(p, st);
+  return cudaErrorInvalidValue;  // lines along y or (one 3D field) z
 }
 
 // Strided passes of N >= 128 take the lines-per-CTA variant p.tl (0 default,
