@@ -32,10 +32,13 @@ template <int N> constexpr int tl_strided(int variant) {
 template <int N, bool CONTIG, int TLV = 0> struct Geo {
   static constexpr int R1 = Plan<N>::R1, R2 = Plan<N>::R2;
   static constexpr int T = R1 < R2 ? R1 : R2;            // threads per line
-  // lines per CTA; strided passes of N = 1024 take 8 lines (64 B runs) so that a
+  // lines per CTA; contiguous passes of N >= 256 take two warps' worth: small CTAs
+  // fill the SM (90 registers: two CTAs of 256 threads, ten of 64) and their loads
+  // and stores overlap (512: 6.06 -> 6.73 TB/s, 1024: 6.08 -> 6.65, 256: 6.81 ->
+  // 7.21 against 256 threads).  Strided passes of N = 1024 take 8 lines (64 B runs) so that a
   // CTA stages 64 KB rather than 128 KB and two CTAs per SM overlap their loads
   // and stores (at N = 512, 16 lines measured faster); TLV selects a variant
-  static constexpr int TL = CONTIG ? (N <= 32 ? 8 : 256 / T) : tl_strided<N>(TLV);
+  static constexpr int TL = CONTIG ? (N <= 32 ? 8 : N >= 256 ? 64 / T : 256 / T) : tl_strided<N>(TLV);
   static constexpr int THREADS = TL * T;
   static constexpr int R2S = CONTIG ? R2 + 1 : R2;       // padded row of Y (contiguous layout)
   static constexpr int LS = CONTIG ? R1 * R2S + 1 : 0;
