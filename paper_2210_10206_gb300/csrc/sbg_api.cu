@@ -414,7 +414,10 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
   //                     into fewer tiles.
   auto half = [&](int b) { return b < (nb + 1) / 2 ? 0 : 1; };
   struct RowKey { int a1, b1, a2, b2; };
-  struct Slab { int r0, nr, c0, nc; long long tout; int row0, tile; };
+  // a tile's place in T: entry (r, c) of the block's column chunk is at row pos,
+  // column cpos[c - c0] of the tile
+  struct Slab { int tile, c0; std::vector<int> cpos; };
+  struct Place { int slab = -1, pos = 0; };
   struct Block {
     int m3 = 0, b2 = 0;
     std::vector<RowKey> rows;
@@ -422,7 +425,8 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
     std::vector<int> l3s;
     int ncols = 0, bcol0 = 0;  // columns: b3 in [bcol0, nb) x l3s, b3-major
     std::vector<Slab> slabs;
-    std::vector<std::vector<int>> slab_at;  // [column chunk][row] -> slab
+    std::vector<std::vector<Place>> place;  // [column chunk][row]
+    std::vector<unsigned> used;             // [row] bit i: the output takes entries of column l3s[i]
   };
   auto rkey = [](int a1, int b1, int a2, int b2) -> long long {
     return (((long long)a1 * 64 + b1) * 4096 + a2) * 64 + b2;
@@ -749,140 +753,40 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
       const RowKey& k = bk.rows[r];
       bk.row_of[rkey(k.a1, k.b1, k.a2, k.b2)] = r;
     }
+    bk.used.assign(bk.rows.size(), 0u);
   }
-  long long so = 0;
-  t.tc = tc;
-  for (Block& bk : blocks) {
-    const int nrows_blk = (int)bk.rows.size();
-    if (nrows_blk == 0) continue;
-    for (int c0 = 0; c0 < bk.ncols; c0 += col_chunk) {
-      const int nc = std::min(col_chunk, bk.ncols - c0);
-      const int cls = tc ? 0 : (nc <= 16 ? 0 : (nc <= 32 ? 1 : 2));
-      int TR = 128, tile_u = max_u;
-      SimtGeometry geo{};
-      if (!tc) {
-        // the units of the span grid: rows x columns of 4096 entries, cut in order
-        const int span_rows = cls == 0 ? 256 : (cls == 1 ? 128 : 64);
-        t.simt.span_tiles[cls] += (int)count_tiles(bk.rows, span_rows);
-        // the kernel's tiles
-        geo = simt_geometry(cplx ? 1 : 0, nc);
-        tile_u = geo.max_uniq;
-        TR = geo.max_rows;
-      }
-      const int col0 = (int)t.cols.size();
-      int bgroup = -1;
-      if (tc) {
-        BGroup g{};
-        g.col0 = col0;
-        g.ncols = nc;
-        g.n = ((cplx ? 2 * nc : nc) + 7) & ~7;  // the MMAs take 2n and n rounded up to 16
-        // the kernel's B stage holds 2n rows of 128 bytes and its inner
-        // accumulator 3n TMEM columns: n <= 64
-        if (g.n > 64) return fail(ctx, SBG_ERR_INTERNAL, "tensor-core column group wider than 64");
-        g.off = t.img_stride;
-        t.img_stride += (long long)g.n * 256;
-        t.chunks_per_kb += g.n * 8;
-        bgroup = (int)t.bgroups.size();
-        t.bgroups.push_back(g);
-      }
-      for (int c = c0; c < c0 + nc; ++c) {
-        const int b3 = bk.bcol0 + c / (int)bk.l3s.size();
-        const int l3 = bk.l3s[c % bk.l3s.size()];
-        t.cols.push_back(store_index(dim, nb, l3, bk.m3, b3));
-      }
-      int r = 0;
-      while (r < nrows_blk) {
-        Tile4 tl{};
-        tl.row0 = (int)t.rows.size();
-        tl.col0 = col0;
-        tl.ncols = nc;
-        tl.uniq0 = (int)t.uniq.size();
-        tl.bgroup = bgroup;
-        std::map<int, int> local;
-        int nr = 0;
-        const int rstart = r;
-        while (r < nrows_blk && nr < TR) {
-          const RowKey rk = bk.rows[r];
-          const Ang a1 = angs[rk.a1], a2 = angs[rk.a2];
-          const int s1 = store_index(dim, nb, a1.l, std::abs(a1.m), rk.b1);
-          const int s2 = store_index(dim, nb, a2.l, std::abs(a2.m), rk.b2);
-          const int need = (local.count(s1) ? 0 : 1) + ((local.count(s2) || s2 == s1) ? 0 : 1);
-          if ((int)local.size() + need > tile_u) break;
-          if (!local.count(s1)) { const int k = (int)local.size(); local[s1] = k; if (!tc) t.uniq.push_back(s1); }
-          if (!local.count(s2)) { const int k = (int)local.size(); local[s2] = k; if (!tc) t.uniq.push_back(s2); }
-          Row4 rw;
-          rw.u1 = local[s1];
-          rw.u2 = local[s2];
-          rw.flags = (a1.m < 0 ? 1 : 0) | (a2.m < 0 ? 2 : 0);
-          float sg = 1.0f;
-          if (dim == 3) {
-            if (a1.m < 0 && (std::abs(a1.m) & 1)) sg = -sg;
-            if (a2.m < 0 && (std::abs(a2.m) & 1)) sg = -sg;
-          }
-          rw.sign = sg;
-          t.rows.push_back(rw);
-          ++nr;
-          ++r;
-        }
-        if (nr == 0) return fail(ctx, SBG_ERR_INTERNAL, "4PCF tiling: a row needs more staged singles than allowed");
-        tl.nrows = nr;
-        tl.nuniq = (int)local.size();
-        if (tc) ST(colour_slots(ctx, t, tl, local));
-        tl.tout = so;
-        if ((int)bk.slab_at.size() <= c0 / col_chunk) bk.slab_at.resize(c0 / col_chunk + 1);
-        bk.slab_at[c0 / col_chunk].resize(nrows_blk, -1);
-        for (int q = rstart; q < rstart + nr; ++q) bk.slab_at[c0 / col_chunk][q] = (int)bk.slabs.size();
-        bk.slabs.push_back({rstart, nr, c0, nc, so, tl.row0, (int)t.tiles.size()});
-        if (tc) {
-          so += (long long)nr * nc;
-        } else {
-          tl.cls = cls;
-          tl.nrg = (nr + geo.rt - 1) / geo.rt;
-          tl.ncg = geo.ncg;
-          so += (long long)geo.rt * geo.ct * tl.nrg * tl.ncg;
-          const int k = geo.ct == 8 ? 1 : 0;
-          t.simt.threads[k] = std::max(t.simt.threads[k], tl.nrg * tl.ncg);
-          t.simt.smem[k] = std::max(t.simt.smem[k], simt_tile_smem(tl, geo));
-          t.simt.uses[k][cls] = true;
-          ++t.simt.ntiles[k];
-        }
-        t.tiles.push_back(tl);
-      }
-    }
-  }
-  t.tcount = so;
-
-  // T index of a triple of singles (any order, any sign of M); negative when the
-  // entry found is the conjugate (all m negated).  rowsign receives the sign the
-  // contraction kernels leave out of that entry's row.
-  auto find_entry = [&](const Single& x, const Single& y, const Single& z, bool neg, float* rowsign) -> long long {
+  // The sign of a row's pair, a_{l,-m} = (-1)^m conj(a_lm) (3D): the FP32 kernel
+  // leaves it to the couplings
+  auto row_sign = [&](const RowKey& k) {
+    return dim == 3 && (((angs[k.a1].m < 0 && (angs[k.a1].m & 1)) != (angs[k.a2].m < 0 && (angs[k.a2].m & 1)))) ? -1.0f
+                                                                                                          : 1.0f;
+  };
+  // Entry of a triple of singles (any order, any sign of M): its block, row and
+  // column; neg: the entry is the conjugate's (all m negated).  rowsign receives
+  // its row's sign.
+  struct Entry { int block = -1, row = 0, col = 0; bool neg = false; };
+  auto find_entry = [&](const Single& x, const Single& y, const Single& z, bool neg, float* rowsign) -> Entry {
     const int m3 = z.m;
-    if (m3 < 0 || m3 > L) return LLONG_MIN;
-    if (x.m + y.m != -m3) return LLONG_MIN;
+    if (m3 < 0 || m3 > L) return {};
+    if (x.m + y.m != -m3) return {};
     const int bi = block_of(m3, tc ? 0 : y.b);
-    if (bi < 0 || bi >= (int)blocks.size()) return LLONG_MIN;
-    const Block& bk = blocks[bi];
+    if (bi < 0 || bi >= (int)blocks.size()) return {};
+    Block& bk = blocks[bi];
     int i1 = ang_index(x.l, x.m), i2 = ang_index(y.l, y.m);
     int b1 = x.b, b2 = y.b;
     if (uniform && b1 == b2 && i2 < i1) std::swap(i1, i2);
     auto it = bk.row_of.find(rkey(i1, b1, i2, b2));
-    if (it == bk.row_of.end()) return LLONG_MIN;
+    if (it == bk.row_of.end()) return {};
     const int row = it->second;
-    if (z.b < bk.bcol0) return LLONG_MIN;
+    if (z.b < bk.bcol0) return {};
     const int l3pos = dim == 3 ? z.l - m3 : 0;
     const int col = (z.b - bk.bcol0) * (int)bk.l3s.size() + l3pos;
-    const int chunk = col / col_chunk;
-    if (col >= bk.ncols || chunk >= (int)bk.slab_at.size() || bk.slab_at[chunk][row] < 0) return LLONG_MIN;
-    const Slab& sl = bk.slabs[bk.slab_at[chunk][row]];
-    long long ti = sl.tout + (long long)(row - sl.r0) * sl.nc + (col - sl.c0);
-    if (!tc) {
-      const Tile4& tl = t.tiles[sl.tile];
-      ti = simt_entry(tl, simt_geometry(cplx ? 1 : 0, tl.ncols), row - sl.r0, col - sl.c0);
-    }
-    if (rowsign) *rowsign = t.rows[sl.row0 + (row - sl.r0)].sign;
-    return neg ? -ti - 1 : ti;
+    if (col >= bk.ncols) return {};
+    bk.used[row] |= 1u << l3pos;
+    if (rowsign) *rowsign = row_sign(bk.rows[row]);
+    return {bi, row, col, neg};
   };
-  auto lookup = [&](Single s[3], float* rowsign) -> long long {
+  auto lookup = [&](Single s[3], float* rowsign) -> Entry {
     static const int perms[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
     for (int neg = 0; neg < 2; ++neg)
       for (const auto& p : perms) {
@@ -890,13 +794,18 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
         if (neg) { x.m = -x.m; y.m = -y.m; z.m = -z.m; }
         if (x.b > y.b) continue;
         if (!uniform && z.b < y.b) continue;
-        const long long ti = find_entry(x, y, z, neg != 0, rowsign);
-        if (ti != LLONG_MIN) return ti;
+        const Entry e = find_entry(x, y, z, neg != 0, rowsign);
+        if (e.block >= 0) return e;
       }
-    return LLONG_MIN;
+    return {};
   };
 
   // coupling CSR: one output per (Lambda, b1, b2, b3) [3D] or (m1, m2, b1, b2, b3) [2D]
+  // (entries: block, row, column and conjugation, turned into T indices once the tiles are cut)
+  std::vector<uint64_t> entries;
+  auto pack_entry = [](const Entry& e) {
+    return (uint64_t)e.block << 48 | (uint64_t)e.row << 20 | (uint64_t)e.col << 1 | (uint64_t)e.neg;
+  };
   t.ptr.clear();
   t.idx.clear();
   t.coef.clear();
@@ -923,17 +832,15 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
                 for (const Term& tm : terms) {
                   Single sg[3] = {{l1, tm.m1, b1}, {l2, tm.m2, b2}, {l3, -(tm.m1 + tm.m2), b3}};
                   float rs = 1.0f;
-                  long long ti = lookup(sg, &rs);
-                  if (ti == LLONG_MIN) return fail(ctx, SBG_ERR_INTERNAL, "4PCF table lookup failed");
-                  double sgn = 1.0;
-                  if (ti < 0) {  // the entry with every m negated holds the conjugate:
-                    ti = -ti - 1;  // Re T is the same, Im T (odd Lambda) changes sign
-                    if (odd) sgn = -1.0;
-                  }
-                  t.idx.push_back((int)ti);
+                  const Entry e = lookup(sg, &rs);
+                  if (e.block < 0) return fail(ctx, SBG_ERR_INTERNAL, "4PCF table lookup failed");
+                  // the entry with every m negated holds the conjugate: Re T is
+                  // the same, Im T (odd Lambda) changes sign
+                  const double sgn = e.neg && odd ? -1.0 : 1.0;
+                  entries.push_back(pack_entry(e));
                   t.coef.push_back(sgn * tm.c * rs);
                 }
-                t.ptr.push_back((int)t.idx.size());
+                t.ptr.push_back((int)entries.size());
               }
         }
   } else {
@@ -945,13 +852,192 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
               const int m3 = -(m1 + m2);
               if (std::abs(m3) <= L) {
                 Single sg[3] = {{-1, m1, b1}, {-1, m2, b2}, {-1, m3, b3}};
-                long long ti = lookup(sg, nullptr);
-                if (ti == LLONG_MIN) return fail(ctx, SBG_ERR_INTERNAL, "2D 4PCF table lookup failed");
-                t.idx.push_back((int)ti);
+                const Entry e = lookup(sg, nullptr);
+                if (e.block < 0) return fail(ctx, SBG_ERR_INTERNAL, "2D 4PCF table lookup failed");
+                entries.push_back(pack_entry(e));
                 t.coef.push_back(1.0);
               }
-              t.ptr.push_back((int)t.idx.size());
+              t.ptr.push_back((int)entries.size());
             }
+  }
+  long long so = 0;
+  t.tc = tc;
+  // A tile: rows `of` rows[r ..] and the columns of `cpos` >= 0, at most TR rows
+  // and tile_u singles.  Returns the rows taken, 0 if none fits.
+  auto cut_tile = [&](Block& bk, const std::vector<int>& rows, size_t r, int TR, int tile_u, Tile4& tl,
+                      std::map<int, int>& local) -> int {
+    tl.row0 = (int)t.rows.size();
+    tl.uniq0 = (int)t.uniq.size();
+    int nr = 0;
+    for (; r < rows.size() && nr < TR; ++r, ++nr) {
+      const RowKey rk = bk.rows[rows[r]];
+      const Ang a1 = angs[rk.a1], a2 = angs[rk.a2];
+      const int s1 = store_index(dim, nb, a1.l, std::abs(a1.m), rk.b1);
+      const int s2 = store_index(dim, nb, a2.l, std::abs(a2.m), rk.b2);
+      const int need = (local.count(s1) ? 0 : 1) + ((local.count(s2) || s2 == s1) ? 0 : 1);
+      if ((int)local.size() + need > tile_u) break;
+      if (!local.count(s1)) { const int k = (int)local.size(); local[s1] = k; if (!tc) t.uniq.push_back(s1); }
+      if (!local.count(s2)) { const int k = (int)local.size(); local[s2] = k; if (!tc) t.uniq.push_back(s2); }
+      Row4 rw;
+      rw.u1 = local[s1];
+      rw.u2 = local[s2];
+      rw.flags = (a1.m < 0 ? 1 : 0) | (a2.m < 0 ? 2 : 0);
+      rw.sign = row_sign(rk);
+      t.rows.push_back(rw);
+    }
+    tl.nrows = nr;
+    tl.nuniq = (int)local.size();
+    return nr;
+  };
+  // FP32 tiles of n rows and nc columns, in entries of the accumulation: the
+  // lanes of their warps, forming the rows (about as long as 10 columns' FMAs)
+  // and about 2000 per tile for staging and barriers
+  auto simt_cost = [&](long long n, int nc) -> double {
+    if (n == 0 || nc == 0) return 0.0;
+    const SimtGeometry g = simt_geometry(cplx ? 1 : 0, nc);
+    auto tile = [&](long long rows) {
+      const long long thr = (rows + g.rt - 1) / g.rt * g.ncg;
+      return (double)((thr + 31) / 32 * 32 * g.rt * g.ct) + 10.0 * rows + 2000.0;
+    };
+    const long long full = n / g.max_rows, rest = n % g.max_rows;
+    return full * tile(g.max_rows) + (rest ? tile(rest) : 0.0);
+  };
+  struct Group { unsigned mask; std::vector<int> rows; };
+  for (Block& bk : blocks) {
+    const int nrows_blk = (int)bk.rows.size();
+    if (nrows_blk == 0) continue;
+    const int nl3 = (int)bk.l3s.size();
+    for (int c0 = 0; c0 < bk.ncols; c0 += col_chunk) {
+      const int nc = std::min(col_chunk, bk.ncols - c0);
+      const int cls = tc ? 0 : (nc <= 16 ? 0 : (nc <= 32 ? 1 : 2));
+      bk.place.push_back(std::vector<Place>(nrows_blk));
+      std::vector<Group> groups;
+      auto columns = [&](unsigned mask) {
+        int n = 0;
+        for (int c = c0; c < c0 + nc; ++c) n += mask >> (c % nl3) & 1;
+        return n;
+      };
+      if (tc) {
+        groups.push_back({~0u, {}});
+        for (int r = 0; r < nrows_blk; ++r) groups[0].rows.push_back(r);
+      } else {
+        // the units of the span grid: rows x columns of 4096 entries, cut in order
+        const int span_rows = cls == 0 ? 256 : (cls == 1 ? 128 : 64);
+        t.simt.span_tiles[cls] += (int)count_tiles(bk.rows, span_rows);
+        t.simt.span_rows += nrows_blk;
+        // The output takes a row's entries of a few l3 only (3D: l1 + l2 + l3 of
+        // one parity within the triangle, and not those another row covers):
+        // the rows of one set of l3 share tiles of its columns, about half of
+        // the block's (lmax 4, 10 bins: 75,500 of 134,320 entries).  Sets too
+        // small to fill their tiles join another one while that costs less.
+        std::map<unsigned, std::vector<int>> sets;
+        for (int r = 0; r < nrows_blk; ++r)
+          if (bk.used[r]) sets[bk.used[r]].push_back(r);
+        for (auto& kv : sets) groups.push_back({kv.first, std::move(kv.second)});
+        for (;;) {
+          double gain = 0.0;
+          size_t ga = 0, gb = 0;
+          for (size_t i = 0; i < groups.size(); ++i)
+            for (size_t j = i + 1; j < groups.size(); ++j) {
+              const Group &p = groups[i], &q = groups[j];
+              const double d = simt_cost(p.rows.size(), columns(p.mask)) + simt_cost(q.rows.size(), columns(q.mask)) -
+                               simt_cost(p.rows.size() + q.rows.size(), columns(p.mask | q.mask));
+              if (d > gain) {
+                gain = d;
+                ga = i;
+                gb = j;
+              }
+            }
+          if (gain <= 0.0) break;
+          groups[ga].mask |= groups[gb].mask;
+          groups[ga].rows.insert(groups[ga].rows.end(), groups[gb].rows.begin(), groups[gb].rows.end());
+          std::sort(groups[ga].rows.begin(), groups[ga].rows.end());
+          groups.erase(groups.begin() + gb);
+        }
+      }
+      for (const Group& gr : groups) {
+        std::vector<int> cpos(nc, -1);
+        const int col0 = (int)t.cols.size();
+        for (int c = c0; c < c0 + nc; ++c) {
+          if (!(gr.mask >> (c % nl3) & 1)) continue;
+          cpos[c - c0] = (int)t.cols.size() - col0;
+          t.cols.push_back(store_index(dim, nb, bk.l3s[c % nl3], bk.m3, bk.bcol0 + c / nl3));
+        }
+        const int gc = (int)t.cols.size() - col0;
+        if (gc == 0) continue;
+        int TR = 128, tile_u = max_u;
+        SimtGeometry geo{};
+        if (!tc) {
+          geo = simt_geometry(cplx ? 1 : 0, gc);
+          tile_u = geo.max_uniq;
+          TR = geo.max_rows;
+        }
+        int bgroup = -1;
+        if (tc) {
+          BGroup g{};
+          g.col0 = col0;
+          g.ncols = gc;
+          g.n = ((cplx ? 2 * gc : gc) + 7) & ~7;  // the MMAs take 2n and n rounded up to 16
+          // the kernel's B stage holds 2n rows of 128 bytes and its inner
+          // accumulator 3n TMEM columns: n <= 64
+          if (g.n > 64) return fail(ctx, SBG_ERR_INTERNAL, "tensor-core column group wider than 64");
+          g.off = t.img_stride;
+          t.img_stride += (long long)g.n * 256;
+          t.chunks_per_kb += g.n * 8;
+          bgroup = (int)t.bgroups.size();
+          t.bgroups.push_back(g);
+        }
+        for (size_t r = 0; r < gr.rows.size();) {
+          Tile4 tl{};
+          tl.col0 = col0;
+          tl.ncols = gc;
+          tl.bgroup = bgroup;
+          std::map<int, int> local;
+          const int nr = cut_tile(bk, gr.rows, r, TR, tile_u, tl, local);
+          if (nr == 0) return fail(ctx, SBG_ERR_INTERNAL, "4PCF tiling: a row needs more staged singles than allowed");
+          if (tc) ST(colour_slots(ctx, t, tl, local));
+          tl.tout = so;
+          for (int q = 0; q < nr; ++q) {
+            Place& pl = bk.place.back()[gr.rows[r + q]];
+            pl.slab = (int)bk.slabs.size();
+            pl.pos = q;
+          }
+          bk.slabs.push_back({(int)t.tiles.size(), c0, cpos});
+          if (tc) {
+            so += (long long)nr * gc;
+          } else {
+            tl.cls = cls;
+            tl.nrg = (nr + geo.rt - 1) / geo.rt;
+            tl.ncg = geo.ncg;
+            so += (long long)geo.rt * geo.ct * tl.nrg * tl.ncg;
+            const int k = geo.ct == 8 ? 1 : 0;
+            t.simt.threads[k] = std::max(t.simt.threads[k], tl.nrg * tl.ncg);
+            t.simt.smem[k] = std::max(t.simt.smem[k], simt_tile_smem(tl, geo));
+            t.simt.uses[k][cls] = true;
+            ++t.simt.ntiles[k];
+          }
+          t.tiles.push_back(tl);
+          r += nr;
+        }
+      }
+    }
+  }
+  t.tcount = so;
+
+  // T indices of the couplings; negative: the entry's conjugate
+  t.idx.resize(entries.size());
+  for (size_t i = 0; i < entries.size(); ++i) {
+    const uint64_t e = entries[i];
+    const Block& bk = blocks[e >> 48];
+    const int row = (int)(e >> 20 & 0xfffffff), col = (int)(e >> 1 & 0x7ffff);
+    const Place& pl = bk.place[col / col_chunk][row];
+    if (pl.slab < 0) return fail(ctx, SBG_ERR_INTERNAL, "4PCF entry without a tile");
+    const Slab& sl = bk.slabs[pl.slab];
+    const Tile4& tl = t.tiles[sl.tile];
+    const int c = sl.cpos[col - sl.c0];
+    long long ti = tl.tout + (long long)pl.pos * tl.ncols + c;
+    if (!tc) ti = simt_entry(tl, simt_geometry(cplx ? 1 : 0, tl.ncols), pl.pos, c);
+    t.idx[i] = (int)(dim == 2 && (e & 1) ? -ti - 1 : ti);
   }
   t.nout = (int)t.ptr.size() - 1;
   if (!tc) {
@@ -2504,7 +2590,7 @@ sbg_status sbg_plan4_info(int dim, int nbins, int lmax, sbg_precision prec, int 
   if (s != SBG_OK) return s;
   if (ntiles)
     *ntiles = t.tc ? (int)t.tiles.size() : t.simt.span_tiles[0] + t.simt.span_tiles[1] + t.simt.span_tiles[2];
-  if (nrows) *nrows = (int)t.rows.size();
+  if (nrows) *nrows = t.tc ? (int)t.rows.size() : t.simt.span_rows;
   if (covering) *covering = t.covering;
   return SBG_OK;
 }

@@ -374,32 +374,34 @@ cudaError_t launch_gram3(const float2* a, long long ng, int nb, const float* del
 // Bound: the FMA pipe (2 FMAs per entry and point, 4 for complex T).  Each thread
 // holds RT rows x CT columns (8 x 8 or 16 x 4 real, 8 x 4 complex: 64
 // accumulators), so a point costs it 6 to 10 16-byte shared-memory loads for 128
-// FMAs.  The FMAs are
-// packed (f32x2, two pipe cycles each), which leaves about half of the issue
-// slots to the loads and to forming the operands.  A packed FMA multiplies two rows
-// by two columns; with the column pair once straight and once swapped in
-// registers it serves the four entries of a 2 x 2 block, and no operand has to
-// be duplicated.  Per 16-point chunk the tile's row singles, its columns and
-// delta are copied with cp.async while the previous chunk is accumulated, then
-// formed in shared memory as [x][row] and [x][column] arrays.  Three to four CTAs of 128 threads per SM overlap one's
-// forming with another's FMAs.
+// FMAs.  The FMAs are packed (f32x2, two pipe cycles each), which leaves about
+// half of the issue slots to the loads and to forming the operands.  A packed FMA
+// multiplies two rows by two columns; with the column pair once straight and once
+// swapped in registers it serves the four entries of a 2 x 2 block, and no operand
+// has to be duplicated.  Per chunk of 8 points (complex T 16) the tile's row
+// singles, its columns and delta are copied with cp.async while the previous chunk
+// is accumulated, then formed in shared memory as [x][row] and [x][column] arrays.
+// Three to four CTAs of 128 threads per SM overlap one's forming with another's
+// FMAs.  The output takes about half of a 3D block's entries (the l3 of one
+// parity), so a tile has few columns (a few l3 of every bin) and up to 512 rows:
+// as many entries per chunk as a wide tile of 16-point chunks.
 // Accumulation: FP32 over a span (at most 512 points), then one FP64 reduction
 // into T (red.add, fire and forget; T is laid out [accumulator][thread], so a
 // warp's 32 values are contiguous): no FP64 add, whose rate is 1/75 of the FMA
 // rate here, occupies the SM.
-// Measured: 256^3, lmax 4, 10 bins: 686 -> 268 ms per field (128^3: 3D lmax 3, 8
-// bins 20.1 -> 8.0 ms; 1024^2, mmax 5, 20 bins 41.4 -> 15.0 ms) against the
-// earlier 4 x 4 entries per thread with two 256-thread CTAs per SM, whose
-// strided float4 loads conflicted in the banks.  The FMA pipe is 60% busy (the
-// bare accumulation loop reaches 80% here); the rest is forming the operands,
-// which narrow tiles (few columns per formed row) pay most, and barriers.
-constexpr int kX = 16;          // points per chunk (half a block of the coefficient store)
-constexpr int kSpan = 32;       // chunks per FP32 span
-constexpr int kRawF = 36;       // floats per raw row: Re x0..15, Im x0..15, pad (16-byte multiple)
+// Measured: 256^3, lmax 4, 10 bins: 686 -> 188 ms per field (268 with every column
+// of a block for each of its rows; 196 with 16-point chunks and 192 rows in the 8 x
+// 8 tiles); 128^3, lmax 3, 8 bins 20.1 -> 6.4 ms (8.0; 7.4); 1024^2, mmax 5, 20
+// bins 41.4 -> 15.0 ms, against the earlier 4 x 4 entries per thread with two
+// 256-thread CTAs per SM, whose strided float4 loads conflicted in the banks.
+constexpr int kSpanX = 512;     // points per FP32 span
 constexpr int kSimtThreads = 128;
+constexpr int simt_x(bool cplx) { return cplx ? 16 : 8; }  // points per chunk
 // most rows of a tile and most columns (complex T: 2D, one column per bin)
-constexpr int simt_rows(int rt) { return rt == 16 ? 256 : 192; }
-constexpr int simt_cols(int ct, bool cplx) { return cplx ? 20 : ct == 4 ? 16 : 64; }
+constexpr int simt_rows(bool cplx) { return cplx ? 192 : 512; }
+constexpr int simt_cols(int ct, bool cplx) { return cplx ? 20 : ct == 4 ? 32 : 64; }
+// floats per raw row: Re, Im of a chunk's points, pad (an odd number of 16-byte units: no bank conflicts)
+constexpr int simt_raw(int x) { return 2 * x + 4; }
 
 __device__ __forceinline__ void simt_cp16(void* dst, const void* src) {
   asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
@@ -421,7 +423,7 @@ __device__ __forceinline__ void red_add(double* p, float v) {
 }
 
 // Spans of one column class: x-split k covers the points [k per, (k + 1) per) and
-// consists of nsp spans of kSpan chunks (the last one shorter or empty).
+// consists of nsp spans of kSpanX points (the last one shorter or empty).
 struct SimtSpans {
   int nsplit, nsp;   // x-splits, spans per x-split
   long long per;     // points per x-split
@@ -449,7 +451,8 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const
   extern __shared__ float4 smem4[];
   // row strides of the formed operands (compile-time: the accumulation's loads
   // and the forming's stores take immediate offsets)
-  constexpr int TRS = simt_rows(RT), TCS = simt_cols(CT, CPLX);
+  constexpr int kX = simt_x(CPLX), kRawF = simt_raw(kX), kP = kX / 2;  // kP: 16-byte pieces of a raw row
+  constexpr int TRS = simt_rows(CPLX), TCS = simt_cols(CT, CPLX);
   const int nrg = tl.nrg, ncg = tl.ncg;
   const int TR = RT * nrg, TC = CT * ncg;
   float* Px = reinterpret_cast<float*>(smem4);   // [kX][TRS]
@@ -465,17 +468,17 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const
   const bool active = rg < nrg;
   const int nraw = tl.nuniq + tl.ncols;
 
-  // the chunk's half (16 Re, 16 Im) of the 32-point block of each single: thread
-  // t copies 16 bytes (chunk t % 8 of the 128) of the raw rows t / 8, + nt / 8, ...
-  const int sch = tid & 7;
-  float* const sdst = raw + (tid >> 3) * kRawF + sch * 4;
-  const float* const ssrc = p.astore + (sch & 3) * 4 + (sch >> 2) * 32;
+  // the chunk's part (kX Re, kX Im) of the 32-point block of each single: thread
+  // t copies piece t % kP of the raw rows t / kP, + nt / kP, ...
+  const int sch = tid % kP;
+  float* const sdst = raw + (tid / kP) * kRawF + sch * 4;
+  const float* const ssrc = p.astore + (sch % (kP / 2)) * 4 + (sch / (kP / 2)) * 32;
   auto stage = [&](long long xc) {
     const float* base = ssrc + (xc >> 5) * (long long)p.nsingle * 64 + (xc & 31);
     float* dst = sdst;
-    for (int row = tid >> 3; row < nraw; row += nt >> 3, dst += (nt >> 3) * kRawF)
+    for (int row = tid / kP; row < nraw; row += nt / kP, dst += (nt / kP) * kRawF)
       simt_cp16(dst, base + (long long)sidx[row] * 64);
-    if (tid < 4) simt_cp16(rdel + tid * 4, p.delta + xc + tid * 4);
+    if (tid < kX / 4) simt_cp16(rdel + tid * 4, p.delta + xc + tid * 4);
     asm volatile("cp.async.commit_group;" ::: "memory");
   };
   // The staged chunk's operands, 8 points of a row or column per item.  meta
@@ -483,7 +486,7 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const
   // conjugations (the row's own sign is left to the couplings).  Rows and columns
   // past the tile's repeat its last ones and are never written out.
   auto form = [&]() {
-    for (int i = tid; i < 2 * TR; i += nt) {
+    for (int i = tid; i < kX / 8 * TR; i += nt) {
       const int h = i >= TR ? 8 : 0, r = i >= TR ? i - TR : i;
       const int2 m = meta[r];
       const float* u1 = raw + (m.x & 0xffff) + h;
@@ -513,7 +516,7 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const
       }
     }
     // columns: the last threads first, whose row items are the fewest
-    for (int i = nt - 1 - tid; i < 2 * TC; i += nt) {
+    for (int i = nt - 1 - tid; i < kX / 8 * TC; i += nt) {
       const int h = i >= TC ? 8 : 0, c = i >= TC ? i - TC : i;
       const float* a = raw + (tl.nuniq + min(c, tl.ncols - 1)) * kRawF + h;
       float* o = Cx + h * TCS + c;
@@ -615,9 +618,9 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const
   auto next_span = [&]() {  // the first span from q on that holds points
     for (; q < s1; ++q) {
       const int k = q / sp.nsp;
-      x0 = k * sp.per + (long long)(q - k * sp.nsp) * (kSpan * kX);
+      x0 = k * sp.per + (long long)(q - k * sp.nsp) * kSpanX;
       const long long left = min((k + 1) * sp.per, p.ng) - x0;
-      nc = (int)min(left, (long long)(kSpan * kX)) / kX;
+      nc = (int)min(left, (long long)kSpanX) / kX;
       if (left > 0) return true;
     }
     return false;
@@ -655,8 +658,9 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const
 
 namespace {
 // shared memory of a tile
-size_t simt_smem(int trs, int tcs, int nuniq, int ncols) {
-  return ((size_t)(nuniq + ncols) * (kRawF + 1) + kX + 2 * kX * ((size_t)trs + tcs)) * 4 + (size_t)trs * 8;
+size_t simt_smem(int ct, bool cplx, int nuniq, int ncols) {
+  const int x = simt_x(cplx), trs = simt_rows(cplx), tcs = simt_cols(ct, cplx);
+  return ((size_t)(nuniq + ncols) * (simt_raw(x) + 1) + x + 2 * x * ((size_t)trs + tcs)) * 4 + (size_t)trs * 8;
 }
 constexpr int kSimtSmemMax = 75 * 1024;
 }  // namespace
@@ -690,23 +694,23 @@ static cudaError_t simt4_t(SimtArgs a, const SimtPlan& pl, int k, int nsm, cudaS
 
 SimtGeometry simt_geometry(int complex_t, int ncols) {
   SimtGeometry g;
-  // 4 columns per thread where 8 would leave a quarter of them empty or more
-  // (128^3, lmax 4, 10 bins: 34.0 ms against 35.3 with 8 everywhere; 5 bins 4.5
-  // against 4.7)
+  // 4 columns per thread where 8 would compute 1 / 0.85 times as many or more (12
+  // and 20 columns: a thread of 16 x 4 loads a quarter more operands per FMA than
+  // one of 8 x 8, which costs less than the empty columns)
   const int c8 = (ncols + 7) / 8 * 8, c4 = (ncols + 3) / 4 * 4;
-  g.ct = complex_t || 4 * c4 <= 3 * c8 ? 4 : 8;
+  g.ct = complex_t || 20 * c4 <= 17 * c8 ? 4 : 8;
   g.rt = complex_t ? 8 : 64 / g.ct;
   g.ncg = (ncols + g.ct - 1) / g.ct;
-  // the most row groups that fill their warps well; at most 96 singles and
+  // the most row groups that fill their warps well; max_uniq singles and
   // simt_rows() rows keep a tile's shared memory near a quarter of an SM's
-  const int most = std::min(kSimtThreads / g.ncg, simt_rows(g.rt) / g.rt);
+  const int most = std::min(kSimtThreads / g.ncg, simt_rows(complex_t != 0) / g.rt);
   auto fill = [&](int n) { return n * g.ncg / (double)((n * g.ncg + 31) / 32 * 32); };
   double best = 0.0;
   for (int n = (most + 1) / 2; n <= most; ++n) best = std::max(best, fill(n));
   int n = most;
   while (fill(n) < best - 0.06) --n;
   g.max_rows = g.rt * n;
-  g.max_uniq = 96;
+  g.max_uniq = complex_t ? 96 : 128;
   return g;
 }
 
@@ -718,7 +722,7 @@ long long simt_entry(const Tile4& t, const SimtGeometry& g, int r, int c) {
 }
 
 size_t simt_tile_smem(const Tile4& t, const SimtGeometry& g) {
-  return simt_smem(simt_rows(g.rt), simt_cols(g.ct, g.rt * g.ct == 32), t.nuniq, t.ncols);
+  return simt_smem(g.ct, g.rt * g.ct == 32, t.nuniq, t.ncols);
 }
 
 cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta, const Tile4* tiles,
@@ -777,7 +781,7 @@ cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta,
     SimtSpans& sp = a.sp[c];
     sp.nsplit = (int)ns;
     sp.per = (chunks + ns - 1) / ns * 32;
-    sp.nsp = (int)((sp.per + kSpan * kX - 1) / (kSpan * kX));
+    sp.nsp = (int)((sp.per + kSpanX - 1) / kSpanX);
     sp.unit = 1;
     a.spf[c] = spf[c];
   }

@@ -53,7 +53,7 @@ struct Row4 {
 // for span_tiles units of 4096 entries (at most kSimtSpanUniq singles each) begin.
 constexpr int kSimtSpanUniq = 64;
 struct SimtPlan {
-  int span_tiles[3];
+  int span_tiles[3], span_rows;
   int first[2], ntiles[2];
   int threads[2];      // the most thread positions (nrg ncg) of the launch's tiles
   size_t smem[2];      // the most dynamic shared memory of its tiles

@@ -66,3 +66,14 @@ def test_slab(ctx):
     for i in range(len(cube)):
         d, _ = O.preprocess(cube[i])
         assert _err(z4[i, ..., 0] + 1j * z4[i, ..., 1], O.zeta4_projected(d, edges, mmax)) < TOL
+
+
+@pytest.mark.parametrize("odd", [False, True])
+def test_full_row_tiles(ctx, odd):
+    """Rows past one tile's 512, sets of l3 joined into one tile, rows no output takes."""
+    n, nb, lmax = 16, 10, 4
+    f = synth.lognormal_field(760, (n, n, n), 1.0, -2.0, dtype=np.float64)
+    edges = np.linspace(0.5, 0.46 * n, nb + 1)
+    d, _ = O.preprocess(f)
+    z4 = ctx.full_odd(f, edges, lmax) if odd else ctx.full(f, edges, lmax4=lmax)[1]
+    assert _err(z4, cpp.zeta4_full(d, edges, lmax, odd=odd)) < TOL
