@@ -371,35 +371,35 @@ cudaError_t launch_gram3(const float2* a, long long ng, int nb, const float* del
 // of the 4PCF (Eq. mu of Sec. 2.3, Eq. proj_4pcf_coeff) as an FP32 SIMT GEMM over
 // x with the pair operand formed on chip.
 //
-// Bound: the FMA pipe (2 FMAs per entry and point, 4 for complex T).  Each thread
-// holds RT rows x CT columns (8 x 8 or 16 x 4 real, 8 x 4 complex: 64
-// accumulators), so a point costs it 6 to 10 16-byte shared-memory loads for 128
-// FMAs.  The FMAs are packed (f32x2, two pipe cycles each), which leaves about
+// Bound: the FMA pipe (2 FMAs per entry and point, 4 for complex T) and, in narrow
+// tiles, the shared-memory pipe.  Each thread holds 8 rows x 8 or 4 columns, so a
+// point costs it 8 or 6 16-byte shared-memory loads for 128 or 64 FMAs (complex T:
+// 128).  The FMAs are packed (f32x2, two pipe cycles each), which leaves about
 // half of the issue slots to the loads and to forming the operands.  A packed FMA
 // multiplies two rows by two columns; with the column pair once straight and once
 // swapped in registers it serves the four entries of a 2 x 2 block, and no operand
 // has to be duplicated.  Per chunk of 8 points (complex T 16) the tile's row
 // singles, its columns and delta are copied with cp.async while the previous chunk
 // is accumulated, then formed in shared memory as [x][row] and [x][column] arrays.
-// Three to four CTAs of 128 threads per SM overlap one's forming with another's
+// Three to seven CTAs of 128 threads per SM overlap one's forming with another's
 // FMAs.  The output takes about half of a 3D block's entries (the l3 of one
-// parity), so a tile has few columns (a few l3 of every bin) and up to 512 rows:
-// as many entries per chunk as a wide tile of 16-point chunks.
+// parity), so a tile has few columns (a few l3 of every bin) and up to 256 rows
+// (512 in 8-column threads).
 // Accumulation: FP32 over a span (at most 512 points), then one FP64 reduction
 // into T (red.add, fire and forget; T is laid out [accumulator][thread], so a
 // warp's 32 values are contiguous): no FP64 add, whose rate is 1/75 of the FMA
 // rate here, occupies the SM.
-// Measured: 256^3, lmax 4, 10 bins: 686 -> 188 ms per field (268 with every column
-// of a block for each of its rows; 196 with 16-point chunks and 192 rows in the 8 x
-// 8 tiles); 128^3, lmax 3, 8 bins 20.1 -> 6.4 ms (8.0; 7.4); 1024^2, mmax 5, 20
-// bins 41.4 -> 15.0 ms, against the earlier 4 x 4 entries per thread with two
-// 256-thread CTAs per SM, whose strided float4 loads conflicted in the banks.
+// Measured: 256^3, lmax 4, 10 bins: 686 -> 176 ms per field (268 with every column
+// of a block for each of its rows); 128^3, lmax 3, 8 bins 20.1 -> 5.4 ms (8.0); 1024^2,
+// mmax 5, 20 bins 41.4 -> 14.9 ms, against the earlier 4 x 4 entries per thread with
+// two 256-thread CTAs per SM, whose strided float4 loads conflicted in the banks.
+// In tiles of 8 x 4 the FMA pipe is 50% busy, the shared-memory pipe 68%, issue 53%.
 constexpr int kSpanX = 512;     // points per FP32 span
 constexpr int kSimtThreads = 128;
 constexpr int simt_x(bool cplx) { return cplx ? 16 : 8; }  // points per chunk
 // most rows of a tile and most columns (complex T: 2D, one column per bin)
-constexpr int simt_rows(bool cplx) { return cplx ? 192 : 512; }
-constexpr int simt_cols(int ct, bool cplx) { return cplx ? 20 : ct == 4 ? 32 : 64; }
+constexpr int simt_rows(int ct, bool cplx) { return cplx ? 192 : ct == 4 ? 256 : 512; }
+constexpr int simt_cols(int ct, bool cplx) { return cplx ? 20 : ct == 4 ? 24 : 64; }
 // floats per raw row: Re, Im of a chunk's points, pad (an odd number of 16-byte units: no bank conflicts)
 constexpr int simt_raw(int x) { return 2 * x + 4; }
 
@@ -442,8 +442,42 @@ struct SimtArgs {
   SimtSpans sp[3];
 };
 
-template <int RT, int CT, bool CPLX>
-__global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const SimtArgs p) {
+// Row and column group of a tile's thread.  A 16-byte shared load of a warp takes
+// two cycles if lanes l and l ^ 1 read one address throughout, or l and l ^ 2,
+// and four otherwise, however few addresses there are (measured: lane / 2, lane %
+// 2 and lane / 4 2.1 cycles, lane / 5 and lane % 4 4.0).  So four lanes take two row
+// groups by two column groups: the row operand is shared by l and l ^ 2, the
+// column operand by l and l ^ 1.  What an odd count leaves over comes last.
+__host__ __device__ __forceinline__ void simt_position(int t, int nrg, int ncg, int& rg, int& cg) {
+  const int pc = ncg >> 1, quads = (nrg >> 1) * pc;
+  if (t < 4 * quads) {
+    const int q = t >> 2, rp = q / pc;
+    rg = 2 * rp + (t & 1);
+    cg = 2 * (q - rp * pc) + (t >> 1 & 1);
+    return;
+  }
+  t -= 4 * quads;
+  if (ncg & 1) {  // the last column group
+    if (t < nrg) {
+      rg = t;
+      cg = ncg - 1;
+      return;
+    }
+    t -= nrg;
+  }
+  rg = nrg - 1;  // the last row group
+  cg = t;
+}
+// its inverse
+inline int simt_thread(int rg, int cg, int nrg, int ncg) {
+  const int pc = ncg >> 1, quads = (nrg >> 1) * pc;
+  if (rg < (nrg & ~1) && cg < (ncg & ~1)) return 4 * ((rg >> 1) * pc + (cg >> 1)) + (rg & 1) + 2 * (cg & 1);
+  if (cg >= (ncg & ~1)) return 4 * quads + rg;
+  return 4 * quads + (ncg & 1 ? nrg : 0) + cg;
+}
+
+template <int CT, bool CPLX>
+__global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : CT == 8 ? 4 : 7) simt4_kernel(const SimtArgs p) {
   const Tile4 tl = p.tiles[blockIdx.x];
   const SimtSpans sp = p.sp[tl.cls];
   const int spf = p.spf[tl.cls];
@@ -451,8 +485,8 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const
   extern __shared__ float4 smem4[];
   // row strides of the formed operands (compile-time: the accumulation's loads
   // and the forming's stores take immediate offsets)
-  constexpr int kX = simt_x(CPLX), kRawF = simt_raw(kX), kP = kX / 2;  // kP: 16-byte pieces of a raw row
-  constexpr int TRS = simt_rows(CPLX), TCS = simt_cols(CT, CPLX);
+  constexpr int RT = 8, kX = simt_x(CPLX), kRawF = simt_raw(kX), kP = kX / 2;  // kP: 16-byte pieces of a raw row
+  constexpr int TRS = simt_rows(CT, CPLX), TCS = simt_cols(CT, CPLX);
   const int nrg = tl.nrg, ncg = tl.ncg;
   const int TR = RT * nrg, TC = CT * ncg;
   float* Px = reinterpret_cast<float*>(smem4);   // [kX][TRS]
@@ -464,8 +498,9 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const
   float* rdel = raw + (tl.nuniq + tl.ncols) * kRawF;
   int* sidx = reinterpret_cast<int*>(rdel + kX);  // store index of each raw row, padded to 16
   const int tid = threadIdx.x, nt = blockDim.x;
-  const int cg = tid % ncg, rg = tid / ncg;
-  const bool active = rg < nrg;
+  int rg, cg;
+  simt_position(tid, nrg, ncg, rg, cg);
+  const bool active = tid < nrg * ncg;
   const int nraw = tl.nuniq + tl.ncols;
 
   // the chunk's part (kX Re, kX Im) of the 32-point block of each single: thread
@@ -659,21 +694,21 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : 4) simt4_kernel(const
 namespace {
 // shared memory of a tile
 size_t simt_smem(int ct, bool cplx, int nuniq, int ncols) {
-  const int x = simt_x(cplx), trs = simt_rows(cplx), tcs = simt_cols(ct, cplx);
+  const int x = simt_x(cplx), trs = simt_rows(ct, cplx), tcs = simt_cols(ct, cplx);
   return ((size_t)(nuniq + ncols) * (simt_raw(x) + 1) + x + 2 * x * ((size_t)trs + tcs)) * 4 + (size_t)trs * 8;
 }
 constexpr int kSimtSmemMax = 75 * 1024;
 }  // namespace
 
-template <int RT, int CT, bool CPLX>
+template <int CT, bool CPLX>
 static cudaError_t simt4_t(SimtArgs a, const SimtPlan& pl, int k, int nsm, cudaStream_t st) {
   const size_t smem = pl.smem[k];
   const int threads = (pl.threads[k] + 31) / 32 * 32;
   if (smem > kSimtSmemMax || threads < 32 || threads > kSimtThreads) return cudaErrorInvalidValue;
-  cudaError_t e = ensure_smem_attr<simt4_kernel<RT, CT, CPLX>>(kSimtSmemMax);
+  cudaError_t e = ensure_smem_attr<simt4_kernel<CT, CPLX>>(kSimtSmemMax);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, simt4_kernel<RT, CT, CPLX>, threads, smem)) !=
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, simt4_kernel<CT, CPLX>, threads, smem)) !=
       cudaSuccess)
     return e;
   // spans per CTA: about 8 CTAs per resident slot, so that the last wave costs
@@ -688,22 +723,26 @@ static cudaError_t simt4_t(SimtArgs a, const SimtPlan& pl, int k, int nsm, cudaS
     if (pl.uses[k][c]) rows = std::max<int>(rows, (int)((spans + sp.unit - 1) / sp.unit));
   }
   a.tiles += pl.first[k];
-  simt4_kernel<RT, CT, CPLX><<<dim3((unsigned)pl.ntiles[k], (unsigned)rows), threads, smem, st>>>(a);
+  simt4_kernel<CT, CPLX><<<dim3((unsigned)pl.ntiles[k], (unsigned)rows), threads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
 SimtGeometry simt_geometry(int complex_t, int ncols) {
   SimtGeometry g;
-  // 4 columns per thread where 8 would compute 1 / 0.85 times as many or more (12
-  // and 20 columns: a thread of 16 x 4 loads a quarter more operands per FMA than
-  // one of 8 x 8, which costs less than the empty columns)
-  const int c8 = (ncols + 7) / 8 * 8, c4 = (ncols + 3) / 4 * 4;
-  g.ct = complex_t || 20 * c4 <= 17 * c8 ? 4 : 8;
-  g.rt = complex_t ? 8 : 64 / g.ct;
+  // Up to 24 columns (most 3D tiles: one or two l3 of each bin), 8 x 4 entries per
+  // thread: 72 registers, so that seven CTAs of tiles of at most 256 rows fit an
+  // SM, against four of 8 x 8 (or 16 x 4, which the next line lists), and their
+  // warps are fuller.  128^3, ms: 8 bins, lmax 3 5.4 (6.5), 10 bins, lmax 4 22.0
+  // (23.0), 5 bins, lmax 4 5.0 (5.5 with five CTAs).  Wider tiles are FMA bound
+  // and take 8 x 8 (20 bins, lmax 2, tiles of 40 columns; with 8 x 4 up to 16
+  // columns only 16.9 against 15.6, up to 32 15.6 but 22.5 for 10 bins).
+  g.cplx = complex_t != 0;
+  g.ct = g.cplx || ncols <= 24 ? 4 : 8;
+  g.rt = 8;
   g.ncg = (ncols + g.ct - 1) / g.ct;
   // the most row groups that fill their warps well; max_uniq singles and
-  // simt_rows() rows keep a tile's shared memory near a quarter of an SM's
-  const int most = std::min(kSimtThreads / g.ncg, simt_rows(complex_t != 0) / g.rt);
+  // simt_rows() rows keep a tile's shared memory within the resident CTAs' share of an SM's
+  const int most = std::min(kSimtThreads / g.ncg, simt_rows(g.ct, g.cplx) / g.rt);
   auto fill = [&](int n) { return n * g.ncg / (double)((n * g.ncg + 31) / 32 * 32); };
   double best = 0.0;
   for (int n = (most + 1) / 2; n <= most; ++n) best = std::max(best, fill(n));
@@ -718,11 +757,11 @@ long long simt_entry(const Tile4& t, const SimtGeometry& g, int r, int c) {
   const int pr = r % (4 * t.nrg), pc = c % (4 * t.ncg);  // within the section
   const int ri = r / (4 * t.nrg) * 4 + pr % 4, cj = c / (4 * t.ncg) * 4 + pc % 4;
   const int i = ri / 2, e = ri & 1, j = cj / 2, w = (cj & 1) ^ e;
-  return t.tout + ((long long)((i * (g.ct / 2) + j) * 2 + w) * 2 + e) * (t.nrg * t.ncg) + pr / 4 * t.ncg + pc / 4;
+  return t.tout + ((long long)((i * (g.ct / 2) + j) * 2 + w) * 2 + e) * (t.nrg * t.ncg) + simt_thread(pr / 4, pc / 4, t.nrg, t.ncg);
 }
 
 size_t simt_tile_smem(const Tile4& t, const SimtGeometry& g) {
-  return simt_smem(g.ct, g.rt * g.ct == 32, t.nuniq, t.ncols);
+  return simt_smem(g.ct, g.cplx, t.nuniq, t.ncols);
 }
 
 cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta, const Tile4* tiles,
@@ -789,9 +828,9 @@ cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta,
   for (int k = 0; k < 2; ++k) {
     if (!plan.ntiles[k]) continue;
     cudaError_t e;
-    if (complex_out == 1) e = simt4_t<8, 4, true>(a, plan, k, nsm, st);
-    else if (k == 0) e = simt4_t<16, 4, false>(a, plan, k, nsm, st);
-    else e = simt4_t<8, 8, false>(a, plan, k, nsm, st);
+    if (complex_out == 1) e = simt4_t<4, true>(a, plan, k, nsm, st);
+    else if (k == 0) e = simt4_t<4, false>(a, plan, k, nsm, st);
+    else e = simt4_t<8, false>(a, plan, k, nsm, st);
     if (e != cudaSuccess) return e;
     ++*launches;
   }

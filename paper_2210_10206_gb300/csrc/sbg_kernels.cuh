@@ -63,6 +63,7 @@ struct SimtPlan {
 // rows and most staged row singles.
 struct SimtGeometry {
   int rt, ct, ncg, max_rows, max_uniq;
+  bool cplx;
 };
 SimtGeometry simt_geometry(int complex_t, int ncols);
 // Index in T of entry (row r, column c) of an FP32 tile, which occupies
