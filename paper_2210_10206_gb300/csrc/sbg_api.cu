@@ -1010,7 +1010,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
             tl.nrg = (nr + geo.rt - 1) / geo.rt;
             tl.ncg = geo.ncg;
             so += (long long)geo.rt * geo.ct * tl.nrg * tl.ncg;
-            const int k = geo.ct == 8 ? 1 : 0;
+            const int k = geo.launch;
             t.simt.threads[k] = std::max(t.simt.threads[k], tl.nrg * tl.ncg);
             t.simt.smem[k] = std::max(t.simt.smem[k], simt_tile_smem(tl, geo));
             t.simt.uses[k][cls] = true;
@@ -1042,7 +1042,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
   t.nout = (int)t.ptr.size() - 1;
   if (!tc) {
     // the tiles of each launch together, in the order they were cut
-    std::stable_partition(t.tiles.begin(), t.tiles.end(), [&](const Tile4& x) { return simt_geometry(cplx ? 1 : 0, x.ncols).ct == 4; });
+    std::stable_partition(t.tiles.begin(), t.tiles.end(), [&](const Tile4& x) { return simt_geometry(cplx ? 1 : 0, x.ncols).launch == 0; });
     t.simt.first[1] = t.simt.ntiles[0];
   }
   if (!to_device) return SBG_OK;

@@ -374,28 +374,29 @@ cudaError_t launch_gram3(const float2* a, long long ng, int nb, const float* del
 // Bound: the FMA pipe (2 FMAs per entry and point, 4 for complex T) and, in narrow
 // tiles, the shared-memory pipe.  Each thread holds 8 rows x 8 or 4 columns, so a
 // point costs it 8 or 6 16-byte shared-memory loads for 128 or 64 FMAs (complex T:
-// 128).  The FMAs are packed (f32x2, two pipe cycles each), which leaves about
-// half of the issue slots to the loads and to forming the operands.  A packed FMA
-// multiplies two rows by two columns; with the column pair once straight and once
-// swapped in registers it serves the four entries of a 2 x 2 block, and no operand
-// has to be duplicated.  Per chunk of 8 points (complex T 16) the tile's row
-// singles, its columns and delta are copied with cp.async while the previous chunk
-// is accumulated, then formed in shared memory as [x][row] and [x][column] arrays.
-// Three to seven CTAs of 128 threads per SM overlap one's forming with another's
-// FMAs.  The output takes about half of a 3D block's entries (the l3 of one
-// parity), so a tile has few columns (a few l3 of every bin) and up to 256 rows
-// (512 in 8-column threads).
+// 128; 4 x 4 in narrow tiles).  The FMAs are packed (f32x2, two pipe cycles each),
+// which leaves about half of the issue slots to the loads and to forming the
+// operands.  A packed FMA multiplies two rows by two columns; with the column pair
+// once straight and once swapped in registers it serves the four entries of a 2 x 2
+// block, and no operand has to be duplicated.  Per chunk of 8 points (complex T 16)
+// the tile's row singles, its columns and delta are copied with cp.async while the
+// previous chunk is accumulated, then formed in shared memory as [x][row] and
+// [x][column] arrays.  Three to seven CTAs per SM overlap one's forming with
+// another's FMAs.  The output takes about half of a 3D block's entries (the l3 of
+// one parity), so a tile has few columns (a few l3 of every bin) and up to 256 rows
+// (512 with 8 columns per thread).
 // Accumulation: FP32 over a span (at most 512 points), then one FP64 reduction
 // into T (red.add, fire and forget; T is laid out [accumulator][thread], so a
 // warp's 32 values are contiguous): no FP64 add, whose rate is 1/75 of the FMA
 // rate here, occupies the SM.
 // Measured: 256^3, lmax 4, 10 bins: 686 -> 176 ms per field (268 with every column
 // of a block for each of its rows); 128^3, lmax 3, 8 bins 20.1 -> 5.4 ms (8.0); 1024^2,
-// mmax 5, 20 bins 41.4 -> 14.9 ms, against the earlier 4 x 4 entries per thread with
+// mmax 5, 20 bins 41.4 -> 14.9 ms; 37 slices of 256^2, mmax 5, 5 bins 1.93 -> 1.72 ms
+// with 4 x 4 for complex T; against the earlier 4 x 4 entries per thread with
 // two 256-thread CTAs per SM, whose strided float4 loads conflicted in the banks.
 // In tiles of 8 x 4 the FMA pipe is 50% busy, the shared-memory pipe 68%, issue 53%.
 constexpr int kSpanX = 512;     // points per FP32 span
-constexpr int kSimtThreads = 128;
+constexpr int simt_threads(int rt) { return rt == 4 ? 256 : 128; }
 constexpr int simt_x(bool cplx) { return cplx ? 16 : 8; }  // points per chunk
 // most rows of a tile and most columns (complex T: 2D, one column per bin)
 constexpr int simt_rows(int ct, bool cplx) { return cplx ? 192 : ct == 4 ? 256 : 512; }
@@ -476,8 +477,8 @@ inline int simt_thread(int rg, int cg, int nrg, int ncg) {
   return 4 * quads + (ncg & 1 ? nrg : 0) + cg;
 }
 
-template <int CT, bool CPLX>
-__global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : CT == 8 ? 4 : 7) simt4_kernel(const SimtArgs p) {
+template <int RT, int CT, bool CPLX>
+__global__ void __launch_bounds__(simt_threads(RT), CPLX ? 3 : CT == 8 ? 4 : 7) simt4_kernel(const SimtArgs p) {
   const Tile4 tl = p.tiles[blockIdx.x];
   const SimtSpans sp = p.sp[tl.cls];
   const int spf = p.spf[tl.cls];
@@ -485,7 +486,7 @@ __global__ void __launch_bounds__(kSimtThreads, CPLX ? 3 : CT == 8 ? 4 : 7) simt
   extern __shared__ float4 smem4[];
   // row strides of the formed operands (compile-time: the accumulation's loads
   // and the forming's stores take immediate offsets)
-  constexpr int RT = 8, kX = simt_x(CPLX), kRawF = simt_raw(kX), kP = kX / 2;  // kP: 16-byte pieces of a raw row
+  constexpr int kX = simt_x(CPLX), kRawF = simt_raw(kX), kP = kX / 2;  // kP: 16-byte pieces of a raw row
   constexpr int TRS = simt_rows(CT, CPLX), TCS = simt_cols(CT, CPLX);
   const int nrg = tl.nrg, ncg = tl.ncg;
   const int TR = RT * nrg, TC = CT * ncg;
@@ -700,15 +701,15 @@ size_t simt_smem(int ct, bool cplx, int nuniq, int ncols) {
 constexpr int kSimtSmemMax = 75 * 1024;
 }  // namespace
 
-template <int CT, bool CPLX>
+template <int RT, int CT, bool CPLX>
 static cudaError_t simt4_t(SimtArgs a, const SimtPlan& pl, int k, int nsm, cudaStream_t st) {
   const size_t smem = pl.smem[k];
   const int threads = (pl.threads[k] + 31) / 32 * 32;
-  if (smem > kSimtSmemMax || threads < 32 || threads > kSimtThreads) return cudaErrorInvalidValue;
-  cudaError_t e = ensure_smem_attr<simt4_kernel<CT, CPLX>>(kSimtSmemMax);
+  if (smem > kSimtSmemMax || threads < 32 || threads > simt_threads(RT)) return cudaErrorInvalidValue;
+  cudaError_t e = ensure_smem_attr<simt4_kernel<RT, CT, CPLX>>(kSimtSmemMax);
   if (e != cudaSuccess) return e;
   int per_sm = 0;
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, simt4_kernel<CT, CPLX>, threads, smem)) !=
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, simt4_kernel<RT, CT, CPLX>, threads, smem)) !=
       cudaSuccess)
     return e;
   // spans per CTA: about 8 CTAs per resident slot, so that the last wave costs
@@ -723,7 +724,7 @@ static cudaError_t simt4_t(SimtArgs a, const SimtPlan& pl, int k, int nsm, cudaS
     if (pl.uses[k][c]) rows = std::max<int>(rows, (int)((spans + sp.unit - 1) / sp.unit));
   }
   a.tiles += pl.first[k];
-  simt4_kernel<CT, CPLX><<<dim3((unsigned)pl.ntiles[k], (unsigned)rows), threads, smem, st>>>(a);
+  simt4_kernel<RT, CT, CPLX><<<dim3((unsigned)pl.ntiles[k], (unsigned)rows), threads, smem, st>>>(a);
   return cudaGetLastError();
 }
 
@@ -738,11 +739,16 @@ SimtGeometry simt_geometry(int complex_t, int ncols) {
   // columns only 16.9 against 15.6, up to 32 15.6 but 22.5 for 10 bins).
   g.cplx = complex_t != 0;
   g.ct = g.cplx || ncols <= 24 ? 4 : 8;
-  g.rt = 8;
+  // Complex T: 4 x 4 entries per thread (80 registers instead of 160) where a tile
+  // of 8 x 4 leaves most of its 128 threads idle or its SM short of warps.  512^2,
+  // mmax 5, ms: 4 bins 0.26 -> 0.20, 8 0.47 -> 0.46, 12 1.00 both, 16 2.03 -> 1.98,
+  // but 20 3.69 -> 4.04 (half as many FMAs per operand load).
+  g.rt = g.cplx && ncols <= 16 ? 4 : 8;
+  g.launch = g.cplx ? g.rt == 8 : g.ct == 8;
   g.ncg = (ncols + g.ct - 1) / g.ct;
   // the most row groups that fill their warps well; max_uniq singles and
   // simt_rows() rows keep a tile's shared memory within the resident CTAs' share of an SM's
-  const int most = std::min(kSimtThreads / g.ncg, simt_rows(g.ct, g.cplx) / g.rt);
+  const int most = std::min(simt_threads(g.rt) / g.ncg, simt_rows(g.ct, g.cplx) / g.rt);
   auto fill = [&](int n) { return n * g.ncg / (double)((n * g.ncg + 31) / 32 * 32); };
   double best = 0.0;
   for (int n = (most + 1) / 2; n <= most; ++n) best = std::max(best, fill(n));
@@ -828,9 +834,8 @@ cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta,
   for (int k = 0; k < 2; ++k) {
     if (!plan.ntiles[k]) continue;
     cudaError_t e;
-    if (complex_out == 1) e = simt4_t<4, true>(a, plan, k, nsm, st);
-    else if (k == 0) e = simt4_t<4, false>(a, plan, k, nsm, st);
-    else e = simt4_t<8, false>(a, plan, k, nsm, st);
+    if (complex_out == 1) e = k == 0 ? simt4_t<4, 4, true>(a, plan, k, nsm, st) : simt4_t<8, 4, true>(a, plan, k, nsm, st);
+    else e = k == 0 ? simt4_t<8, 4, false>(a, plan, k, nsm, st) : simt4_t<8, 8, false>(a, plan, k, nsm, st);
     if (e != cudaSuccess) return e;
     ++*launches;
   }

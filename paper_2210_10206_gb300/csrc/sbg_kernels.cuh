@@ -48,9 +48,10 @@ struct Row4 {
   float sign;          // +-1 from a_{l,-m} = (-1)^m conj(a_{lm}) (3D)
 };
 
-// FP32 tiles of one plan, in two launches: [0] those of 4 columns per thread,
-// [1] those of 8.  The FP32 spans of a column class begin where x-splits chosen
-// for span_tiles units of 4096 entries (at most kSimtSpanUniq singles each) begin.
+// FP32 tiles of one plan, in two launches: [0] those of the fewer entries per
+// thread, [1] the others.  The FP32 spans of a column class begin where x-splits
+// chosen for span_tiles units of 4096 entries (every column of a block for each of
+// its span_rows rows, at most kSimtSpanUniq singles each) begin.
 constexpr int kSimtSpanUniq = 64;
 struct SimtPlan {
   int span_tiles[3], span_rows;
@@ -64,6 +65,7 @@ struct SimtPlan {
 struct SimtGeometry {
   int rt, ct, ncg, max_rows, max_uniq;
   bool cplx;
+  int launch;  // of the plan's two
 };
 SimtGeometry simt_geometry(int complex_t, int ncols);
 // Index in T of entry (row r, column c) of an FP32 tile, which occupies
