@@ -402,7 +402,7 @@ def run_gpu(args):
     traffic = profiled_traffic(args.grid) if prec_name == "bf16x3" else None
     roof = {"bound": bound, "achieved": achieved, "peak": peak, "unit": unit, "frac": achieved / peak,
             "traffic": traffic,
-            "kernel": "tc4_kernel" if prec_name != "fp32" else "simt4_kernel (3 launches)",
+            "kernel": "tc4_kernel" if prec_name != "fp32" else "simt4_kernel (2 launches)",
             "peak_source": peak_src, "alg_flops_per_launch": alg_flops, "avg_ms": kernel_ms}
     hbm = peaks.get("hbm_gbs", 6787.9)
     out = {"metric": METRIC, "value": value, "unit": "fields/s", "n_gpus": ws, "steps": args.steps,

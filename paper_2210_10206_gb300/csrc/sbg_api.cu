@@ -377,8 +377,8 @@ sbg_status colour_slots(sbg_context* ctx, Tables4& t, Tile4& tl, const std::map<
 //   tc = false: FP32 SIMT tiles; for each m3 >= 0 and bin b2, rows (alpha1,
 //               b1 <= b2, alpha2) with m1 + m2 = -m3 and cols (b3 >= b2,
 //               l3 >= m3), or the greedy cover below when it computes fewer
-//               entries; rows per tile 256/128/64 by column class, <= 128
-//               staged singles per tile.
+//               entries; of each row the l3 that the couplings take; tiles as
+//               simt_geometry() has them, <= 128 staged singles each.
 //   tc = true : tensor-core tiles of 128 rows (M of the MMA), <= kTcMaxRowSlots
 //               staged singles, <= 64 B-operand rows (2D: 2 per column single);
 //               one block per m3 >= 0 with columns (b3, l3 >= m3).
@@ -758,8 +758,8 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
   // The sign of a row's pair, a_{l,-m} = (-1)^m conj(a_lm) (3D): the FP32 kernel
   // leaves it to the couplings
   auto row_sign = [&](const RowKey& k) {
-    return dim == 3 && (((angs[k.a1].m < 0 && (angs[k.a1].m & 1)) != (angs[k.a2].m < 0 && (angs[k.a2].m & 1)))) ? -1.0f
-                                                                                                          : 1.0f;
+    auto odd_negative = [&](int a) { return angs[a].m < 0 && (angs[a].m & 1); };
+    return dim == 3 && odd_negative(k.a1) != odd_negative(k.a2) ? -1.0f : 1.0f;
   };
   // Entry of a triple of singles (any order, any sign of M): its block, row and
   // column; neg: the entry is the conjugate's (all m negated).  rowsign receives
@@ -862,8 +862,8 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
   }
   long long so = 0;
   t.tc = tc;
-  // A tile: rows `of` rows[r ..] and the columns of `cpos` >= 0, at most TR rows
-  // and tile_u singles.  Returns the rows taken, 0 if none fits.
+  // Appends the block's rows rows[r], rows[r + 1], ... to a tile, at most TR rows
+  // and tile_u singles.  Returns how many it took.
   auto cut_tile = [&](Block& bk, const std::vector<int>& rows, size_t r, int TR, int tile_u, Tile4& tl,
                       std::map<int, int>& local) -> int {
     tl.row0 = (int)t.rows.size();
@@ -1042,7 +1042,8 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
   t.nout = (int)t.ptr.size() - 1;
   if (!tc) {
     // the tiles of each launch together, in the order they were cut
-    std::stable_partition(t.tiles.begin(), t.tiles.end(), [&](const Tile4& x) { return simt_geometry(cplx ? 1 : 0, x.ncols).launch == 0; });
+    std::stable_partition(t.tiles.begin(), t.tiles.end(),
+                          [&](const Tile4& x) { return simt_geometry(cplx ? 1 : 0, x.ncols).launch == 0; });
     t.simt.first[1] = t.simt.ntiles[0];
   }
   if (!to_device) return SBG_OK;
