@@ -414,18 +414,14 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
   //                     into fewer tiles.
   auto half = [&](int b) { return b < (nb + 1) / 2 ? 0 : 1; };
   struct RowKey { int a1, b1, a2, b2; };
-  // a tile's place in T: entry (r, c) of the block's column chunk is at row pos,
-  // column cpos[c - c0] of the tile
-  struct Slab { int tile, c0; std::vector<int> cpos; };
-  struct Place { int slab = -1, pos = 0; };
   struct Block {
     int m3 = 0, b2 = 0;
     std::vector<RowKey> rows;
     std::unordered_map<long long, int> row_of;
     std::vector<int> l3s;
     int ncols = 0, bcol0 = 0;  // columns: b3 in [bcol0, nb) x l3s, b3-major
-    std::vector<Slab> slabs;
-    std::vector<std::vector<Place>> place;  // [column chunk][row]
+    long long first = 0;                    // entry (row, column) is number first + row ncols + column of the plan's
+    std::vector<float> sign;                // [row]
     std::vector<unsigned> used;             // [row] bit i: the output takes entries of column l3s[i]
   };
   auto rkey = [](int a1, int b1, int a2, int b2) -> long long {
@@ -747,46 +743,50 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
       }
     }
   }
-  for (Block& bk : blocks) {
-    bk.row_of.reserve(bk.rows.size() * 2);
-    for (int r = 0; r < (int)bk.rows.size(); ++r) {
-      const RowKey& k = bk.rows[r];
-      bk.row_of[rkey(k.a1, k.b1, k.a2, k.b2)] = r;
-    }
-    bk.used.assign(bk.rows.size(), 0u);
-  }
   // The sign of a row's pair, a_{l,-m} = (-1)^m conj(a_lm) (3D): the FP32 kernel
   // leaves it to the couplings
   auto row_sign = [&](const RowKey& k) {
     auto odd_negative = [&](int a) { return angs[a].m < 0 && (angs[a].m & 1); };
     return dim == 3 && odd_negative(k.a1) != odd_negative(k.a2) ? -1.0f : 1.0f;
   };
-  // Entry of a triple of singles (any order, any sign of M): its block, row and
-  // column; neg: the entry is the conjugate's (all m negated).  rowsign receives
-  // its row's sign.
-  struct Entry { int block = -1, row = 0, col = 0; bool neg = false; };
-  auto find_entry = [&](const Single& x, const Single& y, const Single& z, bool neg, float* rowsign) -> Entry {
+  long long nentries = 0;
+  for (Block& bk : blocks) {
+    bk.row_of.reserve(bk.rows.size() * 2);
+    for (int r = 0; r < (int)bk.rows.size(); ++r) {
+      const RowKey& k = bk.rows[r];
+      bk.row_of[rkey(k.a1, k.b1, k.a2, k.b2)] = r;
+    }
+    bk.first = nentries;
+    nentries += (long long)bk.rows.size() * bk.ncols;
+    bk.used.assign(bk.rows.size(), 0u);
+    bk.sign.reserve(bk.rows.size());
+    for (const RowKey& k : bk.rows) bk.sign.push_back(row_sign(k));
+  }
+  // Entry of a triple of singles (any order, any sign of M): twice its number, plus
+  // one if it is the conjugate's (all m negated); -1: none.  rowsign receives its
+  // row's sign.
+  auto find_entry = [&](const Single& x, const Single& y, const Single& z, bool neg, float* rowsign) -> long long {
     const int m3 = z.m;
-    if (m3 < 0 || m3 > L) return {};
-    if (x.m + y.m != -m3) return {};
+    if (m3 < 0 || m3 > L) return -1;
+    if (x.m + y.m != -m3) return -1;
     const int bi = block_of(m3, tc ? 0 : y.b);
-    if (bi < 0 || bi >= (int)blocks.size()) return {};
+    if (bi < 0 || bi >= (int)blocks.size()) return -1;
     Block& bk = blocks[bi];
     int i1 = ang_index(x.l, x.m), i2 = ang_index(y.l, y.m);
     int b1 = x.b, b2 = y.b;
     if (uniform && b1 == b2 && i2 < i1) std::swap(i1, i2);
     auto it = bk.row_of.find(rkey(i1, b1, i2, b2));
-    if (it == bk.row_of.end()) return {};
+    if (it == bk.row_of.end()) return -1;
     const int row = it->second;
-    if (z.b < bk.bcol0) return {};
+    if (z.b < bk.bcol0) return -1;
     const int l3pos = dim == 3 ? z.l - m3 : 0;
     const int col = (z.b - bk.bcol0) * (int)bk.l3s.size() + l3pos;
-    if (col >= bk.ncols) return {};
+    if (col >= bk.ncols) return -1;
     bk.used[row] |= 1u << l3pos;
-    if (rowsign) *rowsign = row_sign(bk.rows[row]);
-    return {bi, row, col, neg};
+    if (rowsign) *rowsign = bk.sign[row];
+    return 2 * (bk.first + (long long)row * bk.ncols + col) + neg;
   };
-  auto lookup = [&](Single s[3], float* rowsign) -> Entry {
+  auto lookup = [&](Single s[3], float* rowsign) -> long long {
     static const int perms[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
     for (int neg = 0; neg < 2; ++neg)
       for (const auto& p : perms) {
@@ -794,18 +794,15 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
         if (neg) { x.m = -x.m; y.m = -y.m; z.m = -z.m; }
         if (x.b > y.b) continue;
         if (!uniform && z.b < y.b) continue;
-        const Entry e = find_entry(x, y, z, neg != 0, rowsign);
-        if (e.block >= 0) return e;
+        const long long e = find_entry(x, y, z, neg != 0, rowsign);
+        if (e >= 0) return e;
       }
-    return {};
+    return -1;
   };
 
   // coupling CSR: one output per (Lambda, b1, b2, b3) [3D] or (m1, m2, b1, b2, b3) [2D]
-  // (entries: block, row, column and conjugation, turned into T indices once the tiles are cut)
-  std::vector<uint64_t> entries;
-  auto pack_entry = [](const Entry& e) {
-    return (uint64_t)e.block << 48 | (uint64_t)e.row << 20 | (uint64_t)e.col << 1 | (uint64_t)e.neg;
-  };
+  // (entries become T indices once the tiles are cut)
+  std::vector<long long> entries;
   t.ptr.clear();
   t.idx.clear();
   t.coef.clear();
@@ -832,12 +829,12 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
                 for (const Term& tm : terms) {
                   Single sg[3] = {{l1, tm.m1, b1}, {l2, tm.m2, b2}, {l3, -(tm.m1 + tm.m2), b3}};
                   float rs = 1.0f;
-                  const Entry e = lookup(sg, &rs);
-                  if (e.block < 0) return fail(ctx, SBG_ERR_INTERNAL, "4PCF table lookup failed");
+                  const long long e = lookup(sg, &rs);
+                  if (e < 0) return fail(ctx, SBG_ERR_INTERNAL, "4PCF table lookup failed");
                   // the entry with every m negated holds the conjugate: Re T is
                   // the same, Im T (odd Lambda) changes sign
-                  const double sgn = e.neg && odd ? -1.0 : 1.0;
-                  entries.push_back(pack_entry(e));
+                  const double sgn = (e & 1) && odd ? -1.0 : 1.0;
+                  entries.push_back(e);
                   t.coef.push_back(sgn * tm.c * rs);
                 }
                 t.ptr.push_back((int)entries.size());
@@ -852,9 +849,9 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
               const int m3 = -(m1 + m2);
               if (std::abs(m3) <= L) {
                 Single sg[3] = {{-1, m1, b1}, {-1, m2, b2}, {-1, m3, b3}};
-                const Entry e = lookup(sg, nullptr);
-                if (e.block < 0) return fail(ctx, SBG_ERR_INTERNAL, "2D 4PCF table lookup failed");
-                entries.push_back(pack_entry(e));
+                const long long e = lookup(sg, nullptr);
+                if (e < 0) return fail(ctx, SBG_ERR_INTERNAL, "2D 4PCF table lookup failed");
+                entries.push_back(e);
                 t.coef.push_back(1.0);
               }
               t.ptr.push_back((int)entries.size());
@@ -903,6 +900,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
     return full * tile(g.max_rows) + (rest ? tile(rest) : 0.0);
   };
   struct Group { unsigned mask; std::vector<int> rows; };
+  std::vector<int> index(nentries, -1);  // [entry] its place in T
   for (Block& bk : blocks) {
     const int nrows_blk = (int)bk.rows.size();
     if (nrows_blk == 0) continue;
@@ -910,7 +908,6 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
     for (int c0 = 0; c0 < bk.ncols; c0 += col_chunk) {
       const int nc = std::min(col_chunk, bk.ncols - c0);
       const int cls = tc ? 0 : (nc <= 16 ? 0 : (nc <= 32 ? 1 : 2));
-      bk.place.push_back(std::vector<Place>(nrows_blk));
       std::vector<Group> groups;
       auto columns = [&](unsigned mask) {
         int n = 0;
@@ -956,11 +953,11 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
         }
       }
       for (const Group& gr : groups) {
-        std::vector<int> cpos(nc, -1);
+        std::vector<int> gcols;  // the block's columns of the group
         const int col0 = (int)t.cols.size();
         for (int c = c0; c < c0 + nc; ++c) {
           if (!(gr.mask >> (c % nl3) & 1)) continue;
-          cpos[c - c0] = (int)t.cols.size() - col0;
+          gcols.push_back(c);
           t.cols.push_back(store_index(dim, nb, bk.l3s[c % nl3], bk.m3, bk.bcol0 + c / nl3));
         }
         const int gc = (int)t.cols.size() - col0;
@@ -997,12 +994,6 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
           if (nr == 0) return fail(ctx, SBG_ERR_INTERNAL, "4PCF tiling: a row needs more staged singles than allowed");
           if (tc) ST(colour_slots(ctx, t, tl, local));
           tl.tout = so;
-          for (int q = 0; q < nr; ++q) {
-            Place& pl = bk.place.back()[gr.rows[r + q]];
-            pl.slab = (int)bk.slabs.size();
-            pl.pos = q;
-          }
-          bk.slabs.push_back({(int)t.tiles.size(), c0, cpos});
           if (tc) {
             so += (long long)nr * gc;
           } else {
@@ -1016,6 +1007,10 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
             t.simt.uses[k][cls] = true;
             ++t.simt.ntiles[k];
           }
+          for (int q = 0; q < nr; ++q)
+            for (int c = 0; c < gc; ++c)
+              index[bk.first + (long long)gr.rows[r + q] * bk.ncols + gcols[c]] =
+                  (int)(tc ? tl.tout + (long long)q * gc + c : simt_entry(tl, geo, q, c));
           t.tiles.push_back(tl);
           r += nr;
         }
@@ -1024,20 +1019,12 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
   }
   t.tcount = so;
 
-  // T indices of the couplings; negative: the entry's conjugate
+  // T indices of the couplings; 2D, negative: the entry's conjugate
   t.idx.resize(entries.size());
   for (size_t i = 0; i < entries.size(); ++i) {
-    const uint64_t e = entries[i];
-    const Block& bk = blocks[e >> 48];
-    const int row = (int)(e >> 20 & 0xfffffff), col = (int)(e >> 1 & 0x7ffff);
-    const Place& pl = bk.place[col / col_chunk][row];
-    if (pl.slab < 0) return fail(ctx, SBG_ERR_INTERNAL, "4PCF entry without a tile");
-    const Slab& sl = bk.slabs[pl.slab];
-    const Tile4& tl = t.tiles[sl.tile];
-    const int c = sl.cpos[col - sl.c0];
-    long long ti = tl.tout + (long long)pl.pos * tl.ncols + c;
-    if (!tc) ti = simt_entry(tl, simt_geometry(cplx ? 1 : 0, tl.ncols), pl.pos, c);
-    t.idx[i] = (int)(dim == 2 && (e & 1) ? -ti - 1 : ti);
+    const int ti = index[entries[i] >> 1];
+    if (ti < 0) return fail(ctx, SBG_ERR_INTERNAL, "4PCF entry without a tile");
+    t.idx[i] = dim == 2 && (entries[i] & 1) ? -ti - 1 : ti;
   }
   t.nout = (int)t.ptr.size() - 1;
   if (!tc) {
