@@ -1375,6 +1375,15 @@ sbg_status finish_timings(sbg_context* ctx) {
   return SBG_OK;
 }
 
+// Key of the kernel spectra kept between calls: side, order and the squared edges
+// themselves, all their bits (edges that differ by less than any printed digits can
+// lie on either side of an integer, and then hold other cells).
+std::string spectra_key(int dim, int n, int L, const std::vector<double>& e2) {
+  std::string key = std::to_string(dim) + "/" + std::to_string(n) + "/" + std::to_string(L) + "/";
+  key.append((const char*)e2.data(), e2.size() * sizeof(double));
+  return key;
+}
+
 // Uploads of small host tables are skipped while the device holds the same ones
 // (each costs several microseconds of host time before the first kernel).  A call
 // that fails forgets them: its queued uploads may not have run.
@@ -1494,10 +1503,7 @@ sbg_status measure(sbg_context* ctx, int dim, const void* field, sbg_dtype dtype
   ST(fft_all(ctx, dim, n, -1, LOAD_REAL, d_delta, d_dhat, 1, d_tw));
   rec(ctx, 2);
   // ---- kernel spectra (plan) ----
-  char keyb[512];
-  snprintf(keyb, sizeof keyb, "%d/%d/%d/%d", dim, n, nb, L);
-  std::string key(keyb);
-  for (int i = 0; i <= nb; ++i) key += "/" + std::to_string(e2[i]);
+  const std::string key = spectra_key(dim, n, L, e2);
   const size_t gbytes = (size_t)ngroups * nb * ng * 8;
   const double inv_ng = 1.0 / (double)ng;
   auto gen_group = [&](int g, float2* dst) -> sbg_status {
@@ -1883,10 +1889,7 @@ sbg_status measure_slab(sbg_context* ctx, const sbg_field2d* fields, int nfld, i
   ST(fft_all(ctx, 2, n, -1, LOAD_REAL, d_delta, d_dhat, nfld, d_tw));
   rec(ctx, 2);
   // ---- kernel spectra (shared by the fields: one shape, one bin set) ----
-  char keyb[512];
-  snprintf(keyb, sizeof keyb, "%d/%d/%d/%d", 2, n, nb, mmax);
-  std::string key(keyb);
-  for (int i = 0; i <= nb; ++i) key += "/" + std::to_string(e2[i]);
+  const std::string key = spectra_key(2, n, mmax, e2);
   const size_t gbytes = (size_t)ngroups * nb * ng * 8;
   const double inv_ng = 1.0 / (double)ng;
   auto gen_group = [&](int g, float2* dst) -> sbg_status {
