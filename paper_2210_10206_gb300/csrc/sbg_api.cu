@@ -921,7 +921,6 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
         // the units of the span grid: rows x columns of 4096 entries, cut in order
         const int span_rows = cls == 0 ? 256 : (cls == 1 ? 128 : 64);
         t.simt.span_tiles[cls] += (int)count_tiles(bk.rows, span_rows);
-        t.simt.span_rows += nrows_blk;
         // The output takes a row's entries of a few l3 only (3D: l1 + l2 + l3 of
         // one parity within the triangle, and not those another row covers):
         // the rows of one set of l3 share tiles of its columns, about half of
@@ -2579,9 +2578,8 @@ sbg_status sbg_plan4_info(int dim, int nbins, int lmax, sbg_precision prec, int 
   Tables4 t;
   const sbg_status s = build_tables4(&host, t, dim, nbins, lmax, prec != SBG_PREC_FP32, odd != 0, false);
   if (s != SBG_OK) return s;
-  if (ntiles)
-    *ntiles = t.tc ? (int)t.tiles.size() : t.simt.span_tiles[0] + t.simt.span_tiles[1] + t.simt.span_tiles[2];
-  if (nrows) *nrows = t.tc ? (int)t.rows.size() : t.simt.span_rows;
+  if (ntiles) *ntiles = (int)t.tiles.size();
+  if (nrows) *nrows = (int)t.rows.size();
   if (covering) *covering = t.covering;
   return SBG_OK;
 }

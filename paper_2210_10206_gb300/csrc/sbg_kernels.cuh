@@ -49,12 +49,15 @@ struct Row4 {
 };
 
 // FP32 tiles of one plan, in two launches: [0] those of the fewer entries per
-// thread, [1] the others.  The FP32 spans of a column class begin where x-splits
-// chosen for span_tiles units of 4096 entries (every column of a block for each of
-// its span_rows rows, at most kSimtSpanUniq singles each) begin.
+// thread, [1] the others.  span_tiles counts no tile that is launched: it is the
+// number of units (256, 128 or 64 rows of up to 16, 32 or 64 columns, at most
+// kSimtSpanUniq singles each, every column of a block for each of its rows) for which
+// launch_simt4 chooses the x-splits that its FP32 spans begin at.  Where a span begins
+// sets the rounding of every FP32 result; with a count that does not depend on how the
+// tiles are cut, cutting them otherwise leaves the results' bits as they are.
 constexpr int kSimtSpanUniq = 64;
 struct SimtPlan {
-  int span_tiles[3], span_rows;
+  int span_tiles[3];
   int first[2], ntiles[2];
   int threads[2];      // the most thread positions (nrg ncg) of the launch's tiles
   size_t smem[2];      // the most dynamic shared memory of its tiles

@@ -92,3 +92,15 @@ def test_trimmed_projected_plan(sbg):
     # m3 = 1 was 4 rows over 7 tiles, block m3 = 2 60 rows over 5)
     nt, nr, cov = sbg.sbg_plan4_info(2, 10, 10, sbg.SBG_PREC_BF16X3)
     assert cov == 1 and nt <= 25
+
+
+@pytest.mark.parametrize("dim,nb,lmax,odd,tiles", [(3, 10, 4, 0, 21), (3, 10, 4, 1, 22), (3, 8, 3, 0, 7), (2, 20, 5, 0, 21),
+                                                   (2, 5, 5, 0, 3), (3, 1, 0, 0, 1)])
+def test_fp32_plan_counts_the_launched_tiles(sbg, dim, nb, lmax, odd, tiles):
+    # the tiles of the launched plan, which hold only the columns that the couplings
+    # take of each row (47, 10 and 30 at the first, third and fourth geometry if every
+    # column of a block were computed for each of its rows), of at most 256 rows (3D;
+    # 2D 192)
+    nt, nr, _ = sbg.sbg_plan4_info(dim, nb, lmax, sbg.SBG_PREC_FP32, odd)
+    assert nt == tiles
+    assert nt <= nr <= (256 if dim == 3 else 192) * nt
