@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "sarabande_gb300.h"
+#include "sbg_host.h"
 #include "sbg_kernels.cuh"
 
 using namespace sbg;
@@ -1419,9 +1420,8 @@ sbg_status geometry_tables(sbg_context* ctx, int n, const std::vector<double>& e
   return SBG_OK;
 }
 
-// Copies of results from pinned staging to the caller's arrays, by up to 8 host
-// threads of at least 512 KB each: a fresh result array's page faults cost more
-// than the copy (15.5 MB: 1.5 ms on one thread).
+// Copies of results from pinned staging to the caller's arrays, by as many host
+// threads as copy_threads() gives.
 struct HostCopy {
   void* dst;
   const void* src;
@@ -1438,8 +1438,7 @@ void copy_out(const std::vector<HostCopy>& c) {
       at += x.bytes;
     }
   };
-  const size_t hw = std::max(1u, std::thread::hardware_concurrency());
-  const size_t nt = std::max<size_t>(1, std::min<size_t>({8, hw, total / (512u << 10)}));
+  const size_t nt = copy_threads(total);
   const size_t per = (total / nt + 4095) / 4096 * 4096;
   std::vector<std::thread> th;
   for (size_t t = 1; t < nt; ++t) {
