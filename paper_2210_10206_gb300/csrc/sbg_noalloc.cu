@@ -149,8 +149,8 @@ extern "C" sbg_status sbg_projected3_noalloc(const void* field, sbg_dtype dtype,
   p.in = dhat; p.load = LOAD_COMPLEX; p.outer = N; p.inner = 1;
   NA_CU(fft_axis_pass(N, p, stream));
   // the orders m in steps of as many groups as the scratch arrays hold: every
-  // stage is one launch for all of a step's groups (128^2, 7 bins, mmax 5: 19
-  // launches instead of 47)
+  // stage is one launch for all of a step's groups (128^2, 7 bins, mmax 5, steps of
+  // 5 and 1: 18 kernels instead of 42 and 8 memsets, 298 -> 103 us)
   const int step = std::min(mmax + 1, (int)((long long)kMaxBins * kMaxN * kMaxN / (nbins * ng)));
   for (int m = 0; m <= mmax; m += step) {
     const int k = std::min(step, mmax + 1 - m), arrays = k * nbins;

@@ -49,3 +49,30 @@ def test_noalloc_matches_projected_and_oracle_on_three_calls():
         sbg.sbg_projected3_noalloc(big, [1.0, 2.0], 1, 0, z, stream)
     assert e.value.status == -2
     ctx.close()
+
+
+@pytest.mark.parametrize("n,nb,mmax,steps", [(128, 7, 5, (5, 1)), (256, 3, 10, (3, 3, 3, 2)), (256, 10, 2, (1, 1, 1)),
+                                             (8, 2, 10, (11,)), (8, 10, 3, (4,))])
+def test_noalloc_steps(n, nb, mmax, steps):
+    """The orders m go in steps of as many groups as the scratch arrays (10 of 256^2)
+    hold: several full steps, a shorter last one, steps of one order, the smallest side."""
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2210_10206_gb300 import build, sbg
+    build.build()
+    step = min(mmax + 1, 10 * 256 * 256 // (nb * n * n))
+    assert sum(steps) == mmax + 1 and all(s == step for s in steps[:-1]) and 1 <= steps[-1] <= step
+    edges = np.linspace(0.5, 0.46 * n, nb + 1)
+    f = synth.lognormal_field(90 + nb, (n, n), 1.0, -2.0, dtype=np.float64)
+    d = torch.from_numpy(f).to(device="cuda")
+    z = torch.full((mmax + 1, nb, nb, 2), np.nan, dtype=torch.float64, device="cuda")
+    stream = torch.cuda.current_stream().cuda_stream
+    sbg.sbg_projected3_noalloc(d, edges, mmax, sbg.SBG_SUBTRACT_MEAN, z, stream)
+    torch.cuda.synchronize()
+    got = z.cpu().numpy()
+    delta, _ = O.preprocess(f)
+    orc = O.zeta3_projected(delta, edges, mmax)
+    # every order by itself: a step that misses its block shows whatever m = 0 holds
+    for m in range(mmax + 1):
+        assert _err(got[m, ..., 0] + 1j * got[m, ..., 1], orc[m]) < TOL
