@@ -744,8 +744,8 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
       }
     }
   }
-  // The sign of a row's pair, a_{l,-m} = (-1)^m conj(a_lm) (3D): the FP32 kernel
-  // leaves it to the couplings
+  // The sign of a row's pair, a_{l,-m} = (-1)^m conj(a_lm) (3D): the kernels
+  // leave it to the couplings
   auto row_sign = [&](const RowKey& k) {
     auto odd_negative = [&](int a) { return angs[a].m < 0 && (angs[a].m & 1); };
     return dim == 3 && odd_negative(k.a1) != odd_negative(k.a2) ? -1.0f : 1.0f;
@@ -880,7 +880,6 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
       rw.u1 = local[s1];
       rw.u2 = local[s2];
       rw.flags = (a1.m < 0 ? 1 : 0) | (a2.m < 0 ? 2 : 0);
-      rw.sign = row_sign(rk);
       t.rows.push_back(rw);
     }
     tl.nrows = nr;

@@ -498,7 +498,7 @@ __global__ void __launch_bounds__(simt_threads(RT), CPLX ? 3 : CT == 8 ? 4 : 7) 
   int2* meta = reinterpret_cast<int2*>(Cy + kX * TCS);      // [TRS], see below
   float* raw = reinterpret_cast<float*>(meta + TRS);        // [nuniq + ncols][kRawF], then delta [kX]
   float* rdel = raw + (tl.nuniq + tl.ncols) * kRawF;
-  int* sidx = reinterpret_cast<int*>(rdel + kX);  // store index of each raw row, padded to 16
+  int* sidx = reinterpret_cast<int*>(rdel + kX);  // store index of each raw row
   const int tid = threadIdx.x, nt = blockDim.x;
   int rg, cg;
   simt_position(tid, nrg, ncg, rg, cg);

@@ -40,13 +40,13 @@ struct Tile4 {
   int bgroup;          // tensor-core tiles: the B image (column group) of the tile
   int cls;             // FP32 tiles: span class (0: <= 16 columns, 1: <= 32, 2: <= 64)
   int nrg, ncg;        // FP32 tiles: row and column groups (threads) of the tile
-  long long tout;      // offset (in outputs) of this tile's [nrows][ncols] block of T
+  long long tout;      // where the tile's part of T begins (in outputs): tensor-core tiles
+                       // [nrows][ncols], FP32 tiles [accumulator][thread] (simt_entry)
 };
 struct Row4 {
   int u1, u2;          // local (tile) indices of the two singles
   int flags;           // bit0: conj first, bit1: conj second
-  float sign;          // +-1 from a_{l,-m} = (-1)^m conj(a_{lm}) (3D)
-};
+};  // (the sign of a_{l,-m} = (-1)^m conj(a_{lm}) is in the couplings)
 
 // FP32 tiles of one plan, in two launches: [0] those of the fewer entries per
 // thread, [1] the others.  span_tiles counts no tile that is launched: it is the
@@ -76,9 +76,9 @@ SimtGeometry simt_geometry(int complex_t, int ncols);
 long long simt_entry(const Tile4& t, const SimtGeometry& g, int r, int c);
 size_t simt_tile_smem(const Tile4& t, const SimtGeometry& g);
 
-// T[tile][r][c] (+)= sum_x delta * f1 * f2 * a_col: its real part
+// T at entry (tile, r, c) += sum_x delta * f1 * f2 * a_col: its real part
 // (complex_out 0), complex value (1, two doubles per entry) or imaginary part
-// (2).  *launches receives the kernels launched.
+// (2), for the plan's tiles in T's layout of simt_entry.  *launches receives the kernels launched.
 // A slab of nfld fields (ng = nfld x the points of one field): each field is
 // split alike and adds into T + f t_field_stride (doubles).
 cudaError_t launch_simt4(const float2* astore, long long ng, const float* delta, const Tile4* tiles,
