@@ -383,8 +383,7 @@ cudaError_t launch_gram3(const float2* a, long long ng, int nb, const float* del
 // previous chunk is accumulated, then formed in shared memory as [x][row] and
 // [x][column] arrays.  Three to seven CTAs per SM overlap one's forming with
 // another's FMAs.  The output takes about half of a 3D block's entries (the l3 of
-// one parity), so a tile has few columns (a few l3 of every bin) and up to 256 rows
-// (512 with 8 columns per thread).
+// one parity), so a tile has few columns (a few l3 of every bin) and up to 256 rows.
 // Accumulation: FP32 over a span (at most 512 points), then one FP64 reduction
 // into T (red.add, fire and forget; T is laid out [accumulator][thread], so a
 // warp's 32 values are contiguous): no FP64 add, whose rate is 1/75 of the FMA
@@ -400,7 +399,7 @@ constexpr int kSpanX = 512;     // points per FP32 span
 constexpr int simt_threads(int rt) { return rt == 4 ? 256 : 128; }
 constexpr int simt_x(bool cplx) { return cplx ? 16 : 8; }  // points per chunk
 // most rows of a tile and most columns (complex T: 2D, one column per bin)
-constexpr int simt_rows(int ct, bool cplx) { return cplx ? 192 : ct == 4 ? 256 : 512; }
+constexpr int simt_rows(bool cplx) { return cplx ? 192 : 256; }
 constexpr int simt_cols(int ct, bool cplx) { return cplx ? 20 : ct == 4 ? 24 : 64; }
 // floats per raw row: Re, Im of a chunk's points, pad (an odd number of 16-byte units: no bank conflicts)
 constexpr int simt_raw(int x) { return 2 * x + 4; }
@@ -488,7 +487,7 @@ __global__ void __launch_bounds__(simt_threads(RT), CPLX ? 3 : CT == 8 ? 4 : 7) 
   // row strides of the formed operands (compile-time: the accumulation's loads
   // and the forming's stores take immediate offsets)
   constexpr int kX = simt_x(CPLX), kRawF = simt_raw(kX), kP = kX / 2;  // kP: 16-byte pieces of a raw row
-  constexpr int TRS = simt_rows(CT, CPLX), TCS = simt_cols(CT, CPLX);
+  constexpr int TRS = simt_rows(CPLX), TCS = simt_cols(CT, CPLX);
   const int nrg = tl.nrg, ncg = tl.ncg;
   const int TR = RT * nrg, TC = CT * ncg;
   float* Px = reinterpret_cast<float*>(smem4);   // [kX][TRS]
@@ -696,7 +695,7 @@ __global__ void __launch_bounds__(simt_threads(RT), CPLX ? 3 : CT == 8 ? 4 : 7) 
 namespace {
 // shared memory of a tile
 size_t simt_smem(int ct, bool cplx, int nuniq, int ncols) {
-  const int x = simt_x(cplx), trs = simt_rows(ct, cplx), tcs = simt_cols(ct, cplx);
+  const int x = simt_x(cplx), trs = simt_rows(cplx), tcs = simt_cols(ct, cplx);
   return ((size_t)(nuniq + ncols) * (simt_raw(x) + 1) + x + 2 * x * ((size_t)trs + tcs)) * 4 + (size_t)trs * 8;
 }
 constexpr int kSimtSmemMax = 75 * 1024;
@@ -749,7 +748,7 @@ SimtGeometry simt_geometry(int complex_t, int ncols) {
   g.ncg = (ncols + g.ct - 1) / g.ct;
   // the most row groups that fill their warps well; max_uniq singles and
   // simt_rows() rows keep a tile's shared memory within the resident CTAs' share of an SM's
-  const int most = std::min(simt_threads(g.rt) / g.ncg, simt_rows(g.ct, g.cplx) / g.rt);
+  const int most = std::min(simt_threads(g.rt) / g.ncg, simt_rows(g.cplx) / g.rt);
   auto fill = [&](int n) { return n * g.ncg / (double)((n * g.ncg + 31) / 32 * 32); };
   double best = 0.0;
   for (int n = (most + 1) / 2; n <= most; ++n) best = std::max(best, fill(n));
