@@ -565,8 +565,10 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
               if ((int)cov.size() > off) cands.push_back({m3, rk, off, (int)cov.size() - off});
             }
     // lazy greedy: take the candidate with the most uncovered triples (SIMT:
-    // per column of its block; ties: the first enumerated); a popped value
-    // that went stale is pushed back
+    // per column of its block, as if the tiles took all of them; they take the
+    // l3 that are used, and forming a row costs about 10 columns more: see
+    // simt_cost; ties: the first enumerated); a popped value that went stale
+    // is pushed back
     auto value = [&](const Cand& c, int fresh) { return tc ? (double)fresh : (double)fresh / ucols(c.m3); };
     std::vector<char> done(tid.size(), 0);
     long long left = (long long)tid.size();

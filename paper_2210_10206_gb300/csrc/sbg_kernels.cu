@@ -743,6 +743,11 @@ SimtGeometry simt_geometry(int complex_t, int ncols) {
   // of 8 x 4 leaves most of its 128 threads idle or its SM short of warps.  512^2,
   // mmax 5, ms: 4 bins 0.26 -> 0.20, 8 0.47 -> 0.46, 12 1.00 both, 16 2.03 -> 1.98,
   // but 20 3.69 -> 4.04 (half as many FMAs per operand load).
+  // The CTAs per SM cost spills: 4 x 4 complex 92 bytes at 80 registers, 8 x 4 36 at 72,
+  // 8 x 8 8 at 128.  With two CTAs instead of three (118 registers, none spilt) the
+  // complex tiles of 10 columns gain (256^2, 10 bins 0.240 -> 0.215 ms, 37 slices, 5
+  // bins 1.72 -> 1.58) and those of 13 and 16 lose (512^2 1.43 -> 1.54, 1.98 -> 2.16);
+  // with six instead of seven (80 registers, 20 bytes) 8 x 4 is 1% slower.
   g.rt = g.cplx && ncols <= 16 ? 4 : 8;
   g.launch = g.cplx ? g.rt == 8 : g.ct == 8;
   g.ncg = (ncols + g.ct - 1) / g.ct;
