@@ -394,7 +394,7 @@ cudaError_t launch_gram3(const float2* a, long long ng, int nb, const float* del
 // with 4 x 4 for complex T; against the earlier 4 x 4 entries per thread with
 // two 256-thread CTAs per SM, whose strided float4 loads conflicted in the banks.
 // In tiles of 8 x 4 the shared-memory pipe is 81% busy, the FMA pipe 56%, issue 56%
-// (8 x 8: 53%, 62%, 48%; 128^3, lmax 4, 10 bins).
+// (8 x 8: 54%, 62%, 48%; 128^3, lmax 4, 10 bins).
 constexpr int kSpanX = 512;     // points per FP32 span
 constexpr int simt_threads(int rt) { return rt == 4 ? 256 : 128; }
 constexpr int simt_x(bool cplx) { return cplx ? 16 : 8; }  // points per chunk
