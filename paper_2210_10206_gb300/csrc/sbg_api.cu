@@ -855,7 +855,6 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
                 const long long e = lookup(sg, nullptr);
                 if (e < 0) return fail(ctx, SBG_ERR_INTERNAL, "2D 4PCF table lookup failed");
                 entries.push_back(e);
-                t.coef.push_back(1.0);
               }
               t.ptr.push_back((int)entries.size());
             }
@@ -1042,7 +1041,7 @@ sbg_status build_tables4(sbg_context* ctx, Tables4& t, int dim, int nb, int L, b
   ST(upload(ctx, t.d_bgroups, t.bgroups));
   ST(upload(ctx, t.d_ptr, t.ptr));
   ST(upload(ctx, t.d_idx, t.idx));
-  ST(upload(ctx, t.d_coef, t.coef));
+  if (dim == 3) ST(upload(ctx, t.d_coef, t.coef));  // 2D: every coefficient is 1
   return SBG_OK;
 }
 
@@ -1270,7 +1269,7 @@ sbg_status conv_run(sbg_context* ctx, int dim, int n, const FftXf* d_xf, int t0,
   p.batch = nfld * (t1 - t0);
   p.bstride = ng;
   p.sign = +1;
-  p.xf = d_xf + t0;
+  p.xf = astore ? d_xf + t0 : nullptr;
   p.a0 = a0;
   if (nfld > 1) {
     p.nb_per_field = t1 - t0;
@@ -1307,15 +1306,20 @@ sbg_status conv_stored(sbg_context* ctx, int dim, int n, const FftXf* d_xf, cons
   return SBG_OK;
 }
 
-// The table of this call's transforms on the device (kept while it stays the same).
+// The table of the stored groups' transforms, the first ones of t.xf, on the device
+// (kept while it stays the same).  The others need none: they take factor arrays and
+// outputs in order.
 sbg_status conv_upload(sbg_context* ctx, const ConvTable& t, int dim, int nb, int ngroups, int ngroups4, bool pairs_first,
                        FftXf** out) {
-  ST(buf(ctx, "xf", t.xf.size() * sizeof(FftXf), (void**)out));
+  *out = nullptr;
+  if (!t.stored) return SBG_OK;
+  const size_t bytes = t.stored * sizeof(FftXf);
+  ST(buf(ctx, "xf", bytes, (void**)out));
   const std::string key = std::to_string(dim) + "/" + std::to_string(nb) + "/" + std::to_string(ngroups) + "/" +
                           std::to_string(ngroups4) + (pairs_first ? "/p" : "");
   if (ctx->xf_key != key) {
     ctx->xf_key.clear();
-    CU(cudaMemcpyAsync(*out, t.xf.data(), t.xf.size() * sizeof(FftXf), cudaMemcpyHostToDevice, ctx->stream));
+    CU(cudaMemcpyAsync(*out, t.xf.data(), bytes, cudaMemcpyHostToDevice, ctx->stream));
     ctx->xf_key = key;
   }
   return SBG_OK;
@@ -1406,7 +1410,8 @@ sbg_status geometry_tables(sbg_context* ctx, int n, const std::vector<double>& e
   const std::string name = "tw" + std::to_string(n);
   ST(buf(ctx, name.c_str(), n * 8, (void**)tw));
   ST(buf(ctx, "e2", (kMaxBins + 1) * 8, (void**)d_e2));
-  ST(buf(ctx, "vb", kMaxBins * 8, (void**)d_vb));
+  *d_vb = nullptr;
+  if (!vb.empty()) ST(buf(ctx, "vb", kMaxBins * 8, (void**)d_vb));
   if (!ctx->tw_sides.count(n)) {
     const std::vector<float2> t = twiddles(n);
     CU(cudaMemcpyAsync(*tw, t.data(), n * 8, cudaMemcpyHostToDevice, ctx->stream));

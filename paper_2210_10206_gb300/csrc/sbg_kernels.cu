@@ -861,7 +861,7 @@ __global__ void couple_kernel(const double* __restrict__ T, int complex_t, const
     int i = idx[e];
     const bool cj = i < 0;
     if (cj) i = -i - 1;
-    const double c = coef[e];
+    const double c = coef ? coef[e] : 1.0;
     if (complex_t) {
       re += c * T[2LL * i];
       im += c * (cj ? -T[2LL * i + 1] : T[2LL * i + 1]);

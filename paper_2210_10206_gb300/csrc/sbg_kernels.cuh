@@ -161,7 +161,8 @@ struct FusedGroup {
 cudaError_t launch_fused_group(int n, const FusedGroup& g, cudaStream_t st);
 
 // ---- finalisation ----
-// zeta[o] = sum_{e in [ptr[o], ptr[o+1])} coef[e] * T[idx[e]] (idx < 0: conj of T[-idx-1]).
+// zeta[o] = sum_{e in [ptr[o], ptr[o+1])} coef[e] * T[idx[e]] (idx < 0: conj of T[-idx-1];
+// coef null: every coefficient is 1).
 // A slab of nfld fields: field f reads T + f t_stride (entries) and writes zeta + f nout.
 cudaError_t launch_couple(const double* T, int complex_t, const int* ptr, const int* idx, const double* coef,
                           int nout, double* zeta, cudaStream_t st, int nfld = 1, long long t_stride = 0);
